@@ -287,7 +287,7 @@ puro_status_t puro_fp8_linear_wgrad(const puro_fp8_tensor_t *dy_t, const puro_fp
  *   dx = dy * w_t^T     (as puro_fp8_linear_dgrad)
  *   dw = dy_t * x_t^T   (as puro_fp8_linear_wgrad)
  * The two are independent (both need only the quantised output gradient),
- * so when both run as unsplit 256-wide block-scaled GEMMs they share one
+ * so when both run as unsplit block-scaled GEMMs they share one
  * persistent launch: the tiles of the GEMM with the longer reduction first,
  * then the other's.  Where the long tiles do not divide evenly over the CTA
  * pairs, the pairs with one long tile fewer first take about a long tile's
@@ -450,9 +450,9 @@ void puro_set_wait_timeout_ns(uint64_t ns);
 
 /*
  * Tile width of unsplit block-scaled GEMMs (process-wide): 0 (default) lets
- * a per-shape cost model choose; 256 or 224 forces that form.  The 256-wide
- * form shares half of its tensor-memory accumulator between consecutive
- * tiles; the 224-wide form double-buffers it.  Both compute the same
+ * a per-shape cost model choose among 256, 192 and 128; 256 or 224 forces
+ * that form.  The 256-wide form shares half of its tensor-memory accumulator
+ * between consecutive tiles; the others double-buffer it.  Both compute the same
  * products (summation order differs only by tile boundaries, which do not
  * cross the reduction).  Any other value returns PURO_ERR_INVALID_ARG.
  * For tests and tuning; the paper has no counterpart.

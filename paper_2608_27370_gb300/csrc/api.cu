@@ -104,10 +104,19 @@ puro_status_t validate_fp8_gemm(const puro_fp8_tensor_t *a, const puro_fp8_tenso
     return PURO_OK;
 }
 
+// Tile width of an unsplit GEMM: the width forced for block-scaled GEMMs with
+// BF16 output, else the cost model's.
+int tile_width(GemmKind kind, bool accumulate_f32, int64_t M, int64_t N, int64_t K) {
+    const int forced = g_tile_n.load();
+    if (forced) return kind == kGemmFP8Block && !accumulate_f32 ? forced : 256;
+    return choose_tile_n(M, N, kind == kGemmBF16 ? 2 * K : K);
+}
+
 // Validates D = A * B^T and prepares its launch (nothing is enqueued here).
+// width: the tile width of an unsplit GEMM, 0 to choose it.
 puro_status_t prepare_fp8_gemm(const puro_fp8_tensor_t *a, const puro_fp8_tensor_t *b, void *d, void *workspace,
-                               size_t workspace_bytes, int32_t *dev_status, bool accumulate_f32, GemmArgs *gout,
-                               GemmMaps *mout, GemmAction *action) {
+                               size_t workspace_bytes, int32_t *dev_status, bool accumulate_f32, int width,
+                               GemmArgs *gout, GemmMaps *mout, GemmAction *action) {
     const puro_status_t st = validate_fp8_gemm(a, b, d);
     if (st != PURO_OK) return st;
     const int64_t M = a->rows, N = b->rows, K = a->red;
@@ -128,8 +137,7 @@ puro_status_t prepare_fp8_gemm(const puro_fp8_tensor_t *a, const puro_fp8_tensor
     const int sp = choose_splits(M, N, K, false);
     const bool split = sp > 1 && workspace && aligned16(workspace) &&
                        workspace_bytes >= splitk_workspace_bytes(M, N, K, false);
-    const int forced = g_tile_n.load();
-    const int tile_n = (block && !split && !accumulate_f32) ? (forced ? forced : choose_tile_n(M, N, K)) : 256;
+    const int tile_n = split ? 256 : width ? width : tile_width(block ? kGemmFP8Block : kGemmFP8Tensor, accumulate_f32, M, N, K);
 
     GemmMaps m{};
     if (!make_map(&m.a, CU_TENSOR_MAP_DATA_TYPE_UINT8, a->data, K, M, K, kGemmBKBytes, kGemmBM,
@@ -193,14 +201,14 @@ puro_status_t fp8_gemm(const puro_fp8_tensor_t *a, const puro_fp8_tensor_t *b, v
     GemmMaps m{};
     GemmAction action;
     const puro_status_t st =
-        prepare_fp8_gemm(a, b, d, workspace, workspace_bytes, dev_status, accumulate_f32, &g, &m, &action);
+        prepare_fp8_gemm(a, b, d, workspace, workspace_bytes, dev_status, accumulate_f32, 0, &g, &m, &action);
     if (st != PURO_OK) return st;
     return run_fp8_gemm(action, g, m, static_cast<cudaStream_t>(stream));
 }
 
 // How a linear's backward (Dgrad dX [M, K] over N, Wgrad dW [N, K] over M,
 // block-scaled) runs, given `ws` usable workspace bytes: one grouped launch
-// when both GEMMs are 256-wide and unsplit -- or when the Wgrad would split
+// when both GEMMs are unsplit -- or when the Wgrad would split
 // its reduction but one grouped launch with it unsplit is modelled faster --
 // else each GEMM on its own (a split Wgrad adds its reduction kernel).
 struct BackwardPlan {
@@ -214,13 +222,9 @@ BackwardPlan plan_backward(int64_t M, int64_t N, int64_t K, size_t ws) {
         const int sp = choose_splits(r, c, red, false);
         return (sp > 1 && ws >= splitk_workspace_bytes(r, c, red, false)) ? sp : 1;
     };
-    auto tile_of = [&](int64_t r, int64_t c, int64_t red) {
-        const int forced = g_tile_n.load();
-        return forced ? forced : choose_tile_n(r, c, red);
-    };
     BackwardPlan b{};
     const int sd = split_of(M, K, N), sw = split_of(N, K, M);
-    if (sd == 1 && tile_of(M, K, N) == 256 && tile_of(N, K, M) == 256) {
+    if (sd == 1 && g_tile_n.load() != 224) {
         if (sw == 1)
             b.grouped = true;
         else
@@ -243,19 +247,23 @@ puro_status_t fp8_backward(const puro_fp8_tensor_t *dy, const puro_fp8_tensor_t 
     GemmArgs gd{}, gw{};
     GemmMaps md{}, mw{};
     GemmAction ad, aw;
-    st = prepare_fp8_gemm(dy, w_t, dx, workspace, workspace_bytes, dev_status, false, &gd, &md, &ad);
-    if (st != PURO_OK) return st;
     const size_t ws_usable = (workspace && aligned16(workspace)) ? workspace_bytes : 0;
     const bool both_block = dy->scaling == PURO_SCALE_BLOCK && dy_t->scaling == PURO_SCALE_BLOCK;
-    const bool unsplit_w = both_block && dy->rows > 0 && dy->red > 0 && w_t->rows > 0 &&
-                           plan_backward(dy->rows, dy->red, w_t->rows, ws_usable).wgrad_unsplit;
-    st = prepare_fp8_gemm(dy_t, x_t, dw, unsplit_w ? nullptr : workspace, unsplit_w ? 0 : workspace_bytes, dev_status,
-                          false, &gw, &mw, &aw);
+    BackwardPlan plan{};
+    if (both_block && dy->rows > 0 && dy->red > 0 && w_t->rows > 0)
+        plan = plan_backward(dy->rows, dy->red, w_t->rows, ws_usable);
+    int width = 0;  // of a grouped launch's tiles
+    if (plan.grouped)
+        width = g_tile_n.load() ? g_tile_n.load() : choose_grouped_tile_n(dy->rows, dy->red, w_t->rows);
+    st = prepare_fp8_gemm(dy, w_t, dx, workspace, workspace_bytes, dev_status, false, width, &gd, &md, &ad);
+    if (st != PURO_OK) return st;
+    st = prepare_fp8_gemm(dy_t, x_t, dw, plan.wgrad_unsplit ? nullptr : workspace,
+                          plan.wgrad_unsplit ? 0 : workspace_bytes, dev_status, false, width, &gw, &mw, &aw);
     if (st != PURO_OK) return st;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const bool grouped = ad == kGemmLaunch && aw == kGemmLaunch && gd.kind == kGemmFP8Block &&
-                         gw.kind == kGemmFP8Block && gd.splits == 1 && gw.splits == 1 && gd.tile_n == 256 &&
-                         gw.tile_n == 256;
+                         gw.kind == kGemmFP8Block && gd.splits == 1 && gw.splits == 1 && gd.tile_n == gw.tile_n &&
+                         gd.tile_n != 224;
     if (grouped)
         return cuda_status(gw.K >= gd.K ? launch_gemm_grouped(gw, mw, gd, md, s) : launch_gemm_grouped(gd, md, gw, mw, s));
     st = run_fp8_gemm(ad, gd, md, s);
@@ -271,11 +279,12 @@ puro_status_t bf16_gemm(const void *a, const void *b, void *d, int64_t M, int64_
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (M == 0 || N == 0) return PURO_OK;
     if (K == 0) return cuda_status(cudaMemsetAsync(d, 0, static_cast<size_t>(M * N) * 2, s));
+    const int tile_n = tile_width(kGemmBF16, false, M, N, K);
     GemmMaps m{};
     if (!make_map(&m.a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, a, K, M, K * 2, kGemmBKBytes / 2, kGemmBM,
                   CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map(&m.b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, b, K, N, K * 2, kGemmBKBytes / 2, kGemmBN / 2,
-                  CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map(&m.b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, b, K, N, K * 2, kGemmBKBytes / 2,
+                  static_cast<uint32_t>(tile_n / 2), CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&m.d, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, d, N, M, N * 2, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B))
         return PURO_ERR_CUDA;
     m.ws = m.d;
@@ -286,7 +295,7 @@ puro_status_t bf16_gemm(const void *a, const void *b, void *d, int64_t M, int64_
     g.M = M;
     g.N = N;
     g.K = K;
-    g.tile_n = 256;
+    g.tile_n = tile_n;
     g.status = dev_status;
     g.wait_timeout_ns = g_wait_timeout_ns.load();
     g.num_sms = sm_count();

@@ -66,7 +66,7 @@ constexpr int kPairM = 2 * kBM;    // rows of A per pair tile
 constexpr int kAtomBytes = kGemmBKBytes;       // one 128-byte swizzle row of K: one k-block of FP8
 constexpr int kAtoms = 2;                      // k-blocks per pipeline stage
 constexpr int kBKBytes = kAtoms * kAtomBytes;  // bytes of K per pipeline stage
-constexpr int kStages = 3;                     // 3-deep operand ring (64 KB / 60 KB per stage)
+constexpr int kRingBytes = 3 * 2 * kBM * kBKBytes;  // operand ring: three stages of the 256-wide form (192 KB)
 constexpr int kStagesPerGroup = 512 / kBKBytes;  // stages per group of four k-blocks (one scale chunk)
 constexpr int kThreads = 256;
 constexpr int kTmemCols = 512;
@@ -95,14 +95,17 @@ struct NoQuantEpiSmem {};
 template <int BN, bool QOUT = false>
 struct GemmSmem {
     static constexpr int kBNHalf = BN / 2;                 // rows of B per CTA
-    static constexpr bool kSfbByHelper = (BN != 256);      // B scale images built by warp 2
+    static constexpr bool kSfbByHelper = (BN == 224);      // B scale images built by warps 2 and 3
+    // as many stages as the ring of the 256-wide form holds: 3 (256, 224, 192) or 4 (128)
+    static constexpr int kStages = kRingBytes / ((kBM + kBNHalf) * kBKBytes);
+    static constexpr int kSfbChunks = BN > 128 ? 2 : 1;    // 128-row scale chunks a tile's rows of B touch
     alignas(1024) uint8_t a[kStages][kAtoms][kBM * kAtomBytes];
     alignas(1024) uint8_t b[kStages][kAtoms][kBNHalf * kAtomBytes];
     alignas(1024) uint8_t epi[4][32 * 128];    // per epilogue warp: 32 rows x 128 bytes
     alignas(128) uint8_t sf_a[kStages][512];   // scale vectors of this CTA's 128 rows of A
     // scale vectors of the tile's rows of B: per stage (TMA, BN = 256) or per
     // slot of the helper's ring (BN = 224); 2 x 512 bytes = two tcgen05.cp images
-    alignas(128) uint8_t sf_b[kSfbByHelper ? kSfbSlots : kStages][1024];
+    alignas(128) uint8_t sf_b[kSfbByHelper ? kSfbSlots : kStages][512 * kSfbChunks];
     uint64_t full[kStages];   // even CTA: both CTAs' copies of a stage landed
     uint64_t empty[kStages];  // both CTAs: the pair MMAs reading a stage are done
     uint64_t tfull[2];        // both CTAs: accumulator complete
@@ -510,6 +513,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                    const GemmParams p) {
     using Smem = GemmSmem<BN, OUT == kGemmOutQuant>;
     constexpr int kBNHalf = Smem::kBNHalf;
+    constexpr int kStages = Smem::kStages;
     constexpr bool kMX = (KIND == kGemmFP8Block);
     constexpr bool kHelper = kMX && Smem::kSfbByHelper;
     constexpr bool kShifted = kMX && BN == 256;         // shared-half accumulators
@@ -521,10 +525,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
     constexpr int kAtomK = kAtomBytes / kElemBytes;     // elements of K per 128-byte atom
     constexpr int kKSteps = kAtomBytes / 32;            // MMAs per atom (32 bytes of K each)
     constexpr uint32_t kStageBytes = (kBM + kBNHalf) * kBKBytes;  // one CTA's operand bytes per stage
-    constexpr uint32_t kSfBytes = kHelper ? 512u : 512u + 1024u;  // one CTA's TMA scale bytes per group
+    constexpr uint32_t kSfBytes = kHelper ? 512u : 512u + 512u * Smem::kSfbChunks;  // one CTA's TMA scale bytes per group
     constexpr bool OUT_F32 = (OUT == kGemmOutF32Partial || OUT == kGemmOutF32Add);
     constexpr bool OUT_Q = (OUT == kGemmOutQuant);
-    static_assert(BN == 256 || (BN == 224 && kMX && OUT == kGemmOutBF16), "the 224-wide form is block-scaled, BF16 out");
+    static_assert(BN == 256 || BN == 192 || BN == 128 || (BN == 224 && kMX && OUT == kGemmOutBF16),
+                  "the 224-wide form is block-scaled, BF16 out");
+    static_assert(OUT != kGemmOutF32Partial || BN == 256, "split reductions run 256-wide");
     static_assert(!OUT_Q || (kMX && BN == 256), "the quantising epilogue is block-scaled and 256-wide");
     static_assert(!kMX || kSfBase + kSfSets * kSfColsPerSet <= kTmemCols, "TMEM budget");
     static_assert(kAccShift + BN <= (kMX ? kSfBase : kTmemCols), "accumulators clear of the scale columns");
@@ -619,8 +625,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                         tma_load_2d_pair(sm.sf_a[stage], msfa, full_bar, 0, (a_row / 128) * kgroups + kg);
                         if constexpr (!kHelper) {
                             tma_load_2d_pair(sm.sf_b[stage], msfb, full_bar, 0, (wu.n0 / 128) * kgroups + kg);
-                            tma_load_2d_pair(sm.sf_b[stage] + 512, msfb, full_bar, 0,
-                                             (wu.n0 / 128 + 1) * kgroups + kg);
+                            if constexpr (Smem::kSfbChunks == 2)
+                                tma_load_2d_pair(sm.sf_b[stage] + 512, msfb, full_bar, 0,
+                                                 (wu.n0 / 128 + 1) * kgroups + kg);
                         }
                     }
                     ++issued;
@@ -666,6 +673,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
             }
             tc_fence_after_sync();
             const uint32_t d_tmem = tmem + static_cast<uint32_t>((local & 1) * kAccShift);
+            // a 192-wide tile starts at row 0 or 64 of its first 128-row scale chunk: 32 rows per column
+            const uint32_t sfb_shift = BN == 192 ? static_cast<uint32_t>(wu.n0 % 128) / 32u : 0u;
 
             for (int kb = wu.kb0; kb < wu.kb1; ++kb) {
                 const bool group_start = kMX && (kb % kStagesPerGroup) == 0;
@@ -688,8 +697,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                             tmem_cp_pair_32x128b_warpx4(tmem + sfa_col,
                                                         smem_desc_plain_16B_rows(smem_u32(sm.sf_a[stage])));
                             tmem_cp_pair_32x128b_warpx4(tmem + sfb_col, smem_desc_plain_16B_rows(smem_u32(sfb_src)));
-                            tmem_cp_pair_32x128b_warpx4(tmem + sfb_col + 4,
-                                                        smem_desc_plain_16B_rows(smem_u32(sfb_src + 512)));
+                            if constexpr (Smem::kSfbChunks == 2)
+                                tmem_cp_pair_32x128b_warpx4(tmem + sfb_col + 4,
+                                                            smem_desc_plain_16B_rows(smem_u32(sfb_src + 512)));
                         }
                     }
 #pragma unroll
@@ -711,7 +721,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                             else if constexpr (KIND == kGemmFP8Tensor)
                                 mma_pair_f8(d_tmem, ad, bd, idesc, acc);
                             else
-                                mma_pair_mxf8(d_tmem, ad, bd, idesc, tmem + sfa_col, tmem + sfb_col, acc);
+                                mma_pair_mxf8(d_tmem, ad, bd, idesc, tmem + sfa_col, tmem + sfb_col + sfb_shift, acc);
                         }
                     }
                     tc_commit_pair_multicast(&sm.empty[stage], 0x3);  // stage reusable in both CTAs
@@ -822,15 +832,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                 // as a split partial or added to D
                 const int row0 = (OUT == kGemmOutF32Partial ? wu.split * p.num_m * kPairM : 0) + m0 + 32 * q;
 #pragma unroll
-                for (int h = 0; h < BN / 128; ++h) {
+                for (int h = 0; h < (BN + 127) / 128; ++h) {
+                    const int nc = h == 0 ? 4 : (BN - 128) / 32;
                     uint32_t r[4][32];
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) tmem_ld_32x32b_x32(t_row + 128 * h + 32 * c, r[c]);
+                    for (int c = 0; c < 4; ++c)
+                        if (c < nc) tmem_ld_32x32b_x32(t_row + 128 * h + 32 * c, r[c]);
                     tmem_ld_wait();
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
                         const int col = n0 + 128 * h + 32 * c;
-                        if (col >= n_out) break;
+                        if (c >= nc || col >= n_out) break;
                         if (lane == 0) bulk_wait_group_read0();
                         __syncwarp();
                         uint8_t *row = stage_buf + 128 * lane;
@@ -860,7 +872,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster_cta_scope(tempty0 + 8u * buf);
             } else {
-                // BF16 tile in two halves of 128 columns (BN = 224: 128 + 96).
+                // BF16 tile in halves of 128 columns (BN = 224: 128 + 96, 192:
+                // 128 + 64, 128: one).
                 // Shifted (block kind, BN = 256): the half in the columns the
                 // next tile's accumulator shares ([128, 256) of tensor
                 // memory) first, and the accumulator released once it is in
@@ -871,9 +884,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                 // halves of the staging tile, so a piece is written while the
                 // previous one is still being stored.
                 const int h_first = kShifted ? ((local & 1) ? 0 : 1) : 0;
-                constexpr int kReleaseAt = kShifted ? 0 : 1;
+                constexpr int kHalves = (BN + 127) / 128;
+                constexpr int kReleaseAt = kShifted ? 0 : kHalves - 1;
 #pragma unroll 1
-                for (int hh = 0; hh < 2; ++hh) {
+                for (int hh = 0; hh < kHalves; ++hh) {
                     const int h = hh ^ h_first;
                     const int nc = h == 0 ? 4 : (BN - 128) / 32;
                     uint32_t r[4][32];
@@ -995,22 +1009,67 @@ int choose_splits(int64_t M, int64_t N, int64_t K, bool bf16) {
     return (best_cost * 100 <= base * 85) ? best : 1;
 }
 
-// Tile width of an unsplit block-scaled GEMM.  Modelled pair time = waves x
-// per-tile cycles, with constants fitted to measured GB300 times of both
-// forms over the C5 and C6 linear shapes: about 163 cycles per pair MMA plus
-// a 600-cycle accumulator hand-off per tile for the 256-wide form, 176 cycles
-// per MMA plus 350 per tile for the 224-wide one (its helpers' scale images
-// slow the issue).  The narrower form has more tiles, so it pays off only
-// where the 256-wide tiles leave a much worse last wave; it is taken only for
-// a modelled gain above 5.5%.  (With the hand-off at 600 cycles the 256-wide
-// form measured faster on every shape of both models.)
+// Modelled cycles of one tile: a pair MMA (32 bytes of K) and the tile's
+// hand-off.  Fitted to GB300 times of the three widths over fifteen shapes from
+// [256, 1536] to [32768, 2048], K = 1536 .. 8960, back to back.  The narrower
+// MMAs are bound by the operands' way into shared memory, not by the tensor
+// pipe (a 128-wide one would take 64 cycles there), so a narrow tile is no
+// faster per column; it pays where it fits the same number of rounds, that is
+// where the 256-wide tiles leave many SM pairs idle.  Block-scaled, us at 256 /
+// 192 / 128: [256, 1536, K 1536] 8.0 / 7.5 / 6.8, [256, 1536, 8960] 25.7 /
+// 23.7 / 22.2, [1024, 2048, 2048] 9.9 / 9.8 / 8.8, [2048, 1536, 1536] 9.3 /
+// 8.7 / 11.1; but [2048, 2048, 2048] 10.8 / 14.8 / 13.5 and [8192, 2048, 2048]
+// 27 / 30 / 37.
+struct TileCost {
+    int width, per_mma, per_tile;
+};
+constexpr TileCost kTileCosts[] = {{256, 147, 600}, {192, 135, 400}, {128, 125, 350}};
+
+static int64_t tile_cycles(const TileCost &c, int64_t red) {
+    return (red + kBKBytes - 1) / kBKBytes * kAtoms * 4 * c.per_mma + c.per_tile;
+}
+static int64_t pair_tiles(int64_t rows, int64_t cols, int64_t width) {
+    return (rows + kPairM - 1) / kPairM * ((cols + width - 1) / width);
+}
+
+// Tile width of an unsplit GEMM with K reduction bytes: rounds of tiles over
+// the SM pairs times a tile's modelled cycles; a narrower width than 256 only
+// for a modelled gain above 3%.
 int choose_tile_n(int64_t M, int64_t N, int64_t K) {
-    const int64_t stages = (K + kBKBytes - 1) / kBKBytes;
-    const int64_t m_tiles = (M + kPairM - 1) / kPairM;
-    auto waves = [&](int64_t bn) { return (m_tiles * ((N + bn - 1) / bn) + kSplitRefPairs - 1) / kSplitRefPairs; };
-    const int64_t c256 = waves(256) * (stages * kAtoms * 4 * 163 + 600);
-    const int64_t c224 = waves(224) * (stages * kAtoms * 4 * 176 + 350);
-    return c224 * 1000 < c256 * 945 ? 224 : 256;
+    int best = 256;
+    int64_t best_cost = 0;
+    for (const TileCost &c : kTileCosts) {
+        const int64_t waves = (pair_tiles(M, N, c.width) + kSplitRefPairs - 1) / kSplitRefPairs;
+        const int64_t cost = waves * tile_cycles(c, K);
+        if (c.width == 256 || cost * 100 < best_cost * 97) {
+            best = c.width;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
+// Tile width of a linear's Dgrad (dX [M, K], reduction N) and Wgrad (dW [N, K],
+// reduction M) in one grouped launch: the modelled makespan of the balanced
+// schedule, the longer reduction's tiles first.  Measured at 256 / 192 / 128,
+// us: (M, N, K) = (256, 1536, 1536) 8.1 / 7.6 / 6.8, (640, 1152, 2560) 9.0 /
+// 9.8 / 10.0, (2048, 2048, 2048) 15.9 / 19.4 / 22.1.
+int choose_grouped_tile_n(int64_t M, int64_t N, int64_t K) {
+    int best = 256;
+    int64_t best_cost = 0;
+    const int64_t P = kSplitRefPairs;
+    for (const TileCost &c : kTileCosts) {
+        const int64_t ud = pair_tiles(M, K, c.width), uw = pair_tiles(N, K, c.width);
+        const int64_t td = tile_cycles(c, N), tw = tile_cycles(c, M);
+        const int64_t u0 = td >= tw ? ud : uw, t0 = std::max(td, tw), u1 = td >= tw ? uw : ud, t1 = std::min(td, tw);
+        const int64_t cost =
+            u0 + u1 <= P ? t0 : std::max((u0 + P - 1) / P * t0, (u0 * t0 + u1 * t1 + P - 1) / P + t1);
+        if (c.width == 256 || cost * 100 < best_cost * 97) {
+            best = c.width;
+            best_cost = cost;
+        }
+    }
+    return best;
 }
 
 int64_t splitk_rows_per_chunk(int64_t M) { return (M + kPairM - 1) / kPairM * kPairM; }
@@ -1111,15 +1170,25 @@ static cudaError_t launch_kind(const GemmArgs &g, const GemmMaps &m, int splits,
     return launch_params<KIND, OUT, BN>(make_params<KIND, OUT, BN>(g, splits), g, m, m, s);
 }
 
+// The unsplit GEMM at the tile width g.tile_n.
+template <int KIND, int OUT>
+static cudaError_t launch_width(const GemmArgs &g, const GemmMaps &m, cudaStream_t s) {
+    switch (g.tile_n) {
+        case 128: return launch_kind<KIND, OUT, 128>(g, m, 1, s);
+        case 192: return launch_kind<KIND, OUT, 192>(g, m, 1, s);
+        default: return launch_kind<KIND, OUT, 256>(g, m, 1, s);
+    }
+}
+
 template <int KIND>
 static cudaError_t launch_split_or_not(const GemmArgs &g, const GemmMaps &m, cudaStream_t s) {
     if constexpr (KIND == kGemmFP8Block)
         if (g.quant_out) return launch_kind<KIND, kGemmOutQuant, 256>(g, m, 1, s);
     if (g.splits <= 1) {
-        if (g.accumulate_f32) return launch_kind<KIND, kGemmOutF32Add, 256>(g, m, 1, s);
+        if (g.accumulate_f32) return launch_width<KIND, kGemmOutF32Add>(g, m, s);
         if constexpr (KIND == kGemmFP8Block)
             if (g.tile_n == 224) return launch_kind<KIND, kGemmOutBF16, 224>(g, m, 1, s);
-        return launch_kind<KIND, kGemmOutBF16, 256>(g, m, 1, s);
+        return launch_width<KIND, kGemmOutBF16>(g, m, s);
     }
     cudaError_t e = launch_kind<KIND, kGemmOutF32Partial, 256>(g, m, g.splits, s);
     if (e != cudaSuccess) return e;
@@ -1136,13 +1205,14 @@ static cudaError_t launch_split_or_not(const GemmArgs &g, const GemmMaps &m, cud
                       reinterpret_cast<uint2 *>(g.out));
 }
 
-// Two block-scaled GEMMs (BF16 output, 256-wide, unsplit) in one persistent
-// launch: g0's tiles first, then g1's (the caller puts the problem with the
-// longer reductions first, so the shorter tiles fill the last round).
-cudaError_t launch_gemm_grouped(const GemmArgs &g0, const GemmMaps &m0, const GemmArgs &g1, const GemmMaps &m1,
-                                cudaStream_t s) {
-    GemmParams p = make_params<kGemmFP8Block, kGemmOutBF16, 256>(g0, 1);
-    const GemmParams q = make_params<kGemmFP8Block, kGemmOutBF16, 256>(g1, 1);
+// Two block-scaled GEMMs (BF16 output, unsplit, the same tile width) in one
+// persistent launch: g0's tiles first, then g1's (the caller puts the problem
+// with the longer reductions first, so the shorter tiles fill the last round).
+template <int BN>
+static cudaError_t launch_grouped_width(const GemmArgs &g0, const GemmMaps &m0, const GemmArgs &g1,
+                                        const GemmMaps &m1, cudaStream_t s) {
+    GemmParams p = make_params<kGemmFP8Block, kGemmOutBF16, BN>(g0, 1);
+    const GemmParams q = make_params<kGemmFP8Block, kGemmOutBF16, BN>(g1, 1);
     p.units0 = p.num_units;
     p.N1 = q.N;
     p.num_m1 = q.num_m;
@@ -1155,7 +1225,16 @@ cudaError_t launch_gemm_grouped(const GemmArgs &g0, const GemmMaps &m0, const Ge
     // the pairs with one long unit fewer first take about a long unit's
     // worth of short ones (rounded)
     p.lead = q.num_kb > 0 ? (2 * p.num_kb + q.num_kb) / (2 * q.num_kb) : 0;
-    return launch_params<kGemmFP8Block, kGemmOutBF16, 256>(p, g0, m0, m1, s);
+    return launch_params<kGemmFP8Block, kGemmOutBF16, BN>(p, g0, m0, m1, s);
+}
+
+cudaError_t launch_gemm_grouped(const GemmArgs &g0, const GemmMaps &m0, const GemmArgs &g1, const GemmMaps &m1,
+                                cudaStream_t s) {
+    switch (g0.tile_n) {
+        case 128: return launch_grouped_width<128>(g0, m0, g1, m1, s);
+        case 192: return launch_grouped_width<192>(g0, m0, g1, m1, s);
+        default: return launch_grouped_width<256>(g0, m0, g1, m1, s);
+    }
 }
 
 // Modelled time, in pipeline stages of one pair, of a linear's Dgrad and
@@ -1180,7 +1259,7 @@ bool grouped_backward_faster(int64_t M, int64_t N, int64_t K, int w_splits) {
 
 cudaError_t launch_gemm(const GemmArgs &g, const GemmMaps &m, cudaStream_t s) {
     switch (g.kind) {
-        case kGemmBF16: return launch_kind<kGemmBF16, kGemmOutBF16, 256>(g, m, 1, s);
+        case kGemmBF16: return launch_width<kGemmBF16, kGemmOutBF16>(g, m, s);
         case kGemmFP8Tensor: return launch_split_or_not<kGemmFP8Tensor>(g, m, s);
         default: return launch_split_or_not<kGemmFP8Block>(g, m, s);
     }

@@ -137,9 +137,9 @@ struct GemmArgs {
     GemmKind kind;
     int a_fmt, b_fmt;            // FP8 formats (0 = E4M3, 1 = E5M2)
     int64_t M, N, K;
-    int tile_n;                  // 256, or 224 (block kind, unsplit; see choose_tile_n)
+    int tile_n;                  // 256, 192 or 128 (see choose_tile_n), or 224 (block kind, BF16 out, forced); split: 256
     // kGemmFP8Block: scale vectors of B (the 224-wide form gathers them
-    // itself; the 256-wide form loads them through GemmMaps::sfb).
+    // itself; the others load them through GemmMaps::sfb).
     const uint8_t *sfb;
     // kGemmFP8Tensor: dequantisation factors of A and B.
     const float *sia, *sib;
@@ -167,9 +167,8 @@ struct GemmArgs {
 // Tensor maps of one GEMM launch.
 //   a:   A [M, K] (128-byte swizzle, box {128 bytes, 128 rows})
 //   b:   B [N, K] (box {128 bytes, tile_n / 2 rows}: half of a tile per CTA)
-//   d:   D [M, N] bf16 (tile_n 256: 128-byte swizzle, box {64, 32};
-//        tile_n 224: 64-byte swizzle, box {32, 32}); with accumulate_f32, the
-//        FP32 main-grad [M, N] (128-byte swizzle, box {32, 32})
+//   d:   D [M, N] bf16 (64-byte swizzle, box {32, 32}); with accumulate_f32,
+//        the FP32 main-grad [M, N] (128-byte swizzle, box {32, 32})
 //   ws:  workspace [splits * splitk_rows_per_chunk(M), N] fp32 (128-byte
 //        swizzle, box {32, 32}); only read when g.splits > 1
 //   sfa, sfb (kGemmFP8Block only): the scale vectors of A / B,
@@ -181,7 +180,7 @@ struct GemmMaps {
 
 cudaError_t launch_gemm(const GemmArgs &g, const GemmMaps &m, cudaStream_t s);
 // Two block-scaled GEMMs with BF16 output in one launch (the Dgrad and Wgrad
-// of one linear): 256-wide tiles, neither reduction split.
+// of one linear): the same tile width (256, 192 or 128), neither reduction split.
 cudaError_t launch_gemm_grouped(const GemmArgs &g0, const GemmMaps &m0, const GemmArgs &g1, const GemmMaps &m1,
                                 cudaStream_t s);
 
@@ -203,9 +202,10 @@ int64_t splitk_rows_per_chunk(int64_t M);  // M rounded up to a whole 256-row pa
 // schedule, Wgrad unsplit) than as two launches with the Wgrad split into
 // w_splits chunks.  Host-only, shape-only.
 bool grouped_backward_faster(int64_t M, int64_t N, int64_t K, int w_splits);
-// Tile width (256 or 224) of an unsplit block-scaled GEMM: modelled waves x
-// per-tile time of the two forms.  Host-only, shape-only.
+// Tile width (256, 192 or 128) of an unsplit GEMM with K reduction bytes, and of
+// a linear's Dgrad and Wgrad in one launch.  Host-only, shape-only.
 int choose_tile_n(int64_t M, int64_t N, int64_t K);
+int choose_grouped_tile_n(int64_t M, int64_t N, int64_t K);
 
 // Tile shape of the GEMM kernel: rows of A per CTA (a CTA pair computes
 // 2 * kGemmBM rows), columns of a tile (rows of B per pair), and the bytes

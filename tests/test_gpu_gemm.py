@@ -282,6 +282,40 @@ def test_grouped_backward_equals_separate_calls(M, N, K):
     assert P.puro_fp8_get_status(status) == 0
 
 
+# Tile widths below 256 (chosen where they take fewer idle SM pairs): 128 at
+# few tiles, 192 at nine rows of tiles; the last tile of a row is cut, and the
+# 192-wide tiles start at row 64 of every other 128-row scale chunk.
+@pytest.mark.parametrize("M,N,K", [(128, 128, 128), (384, 896, 640), (2176, 1408, 384), (2304, 1408, 1152)])
+@pytest.mark.parametrize("main_grad", [False, True])
+def test_block_gemm_narrow_tiles(M, N, K, main_grad):
+    x, w, _ = _inputs(M, N, K, 8000 + M + N + K, t3=True)
+    xq = P.quantize(x, P.E4M3, P.SCALE_BLOCK, P.ROLE_ACT, transpose=False)
+    wq = P.quantize(w, P.E4M3, P.SCALE_BLOCK, P.ROLE_ACT, transpose=False)
+    out = torch.zeros((M, N), dtype=torch.float32 if main_grad else torch.bfloat16, device=DEV)
+    call = P.puro_fp8_linear_wgrad_main_grad if main_grad else P.puro_fp8_linear_fprop
+    call(xq.rowwise, wq.rowwise, out)
+    torch.cuda.synchronize()
+    A, B = (O.dequant_rows_1x128(*par_quantize_rows_1x128(bits(t), P.E4M3), P.E4M3) for t in (x, w))
+    assert_close(out, O.gemm_tn(A, B, 8), "narrow tiles")
+
+
+@pytest.mark.parametrize("M,N,K", [(16, 16, 16), (400, 912, 656), (2128, 1424, 400)])
+@pytest.mark.parametrize("kind", ["tensor", "bf16"])
+def test_dense_gemm_narrow_tiles(M, N, K, kind):
+    x, w, _ = _inputs(M, N, K, 8100 + M + N + K)
+    y = torch.empty((M, N), dtype=torch.bfloat16, device=DEV)
+    if kind == "bf16":
+        P.puro_bf16_linear_fprop(x, w, y, M, N, K)
+        A, B = (O.bf16_to_double(bits(t)) for t in (x, w))
+        ref = O.gemm_tn(A, B, 8)
+    else:
+        xq, wq = (P.quantize(t, P.E4M3, P.SCALE_TENSOR, P.ROLE_ACT) for t in (x, w))
+        P.puro_fp8_linear_fprop(xq.rowwise, wq.rowwise, y)
+        ref = oracle_linear(x, w, torch.zeros((M, N), dtype=torch.bfloat16, device=DEV), P.SCALE_TENSOR)["y"]
+    torch.cuda.synchronize()
+    assert_close(y, ref, kind)
+
+
 # --------------------------------------------------------------------------
 # Several tiles per CTA pair.  The persistent grid holds at most 76 pairs on
 # GB300 (152 SMs), so outputs of 256 or more 256-wide pair tiles make every
