@@ -556,7 +556,10 @@ PURO_API puro_status_t puro_fp8_quantize_rmsnorm(const void *h, int64_t rows, in
         return PURO_ERR_CUDA;
     cudaError_t e = launch_rmsnorm_rstd(static_cast<const uint16_t *>(h), rows, cols, eps, rstd, s);
     if (e != cudaSuccess) return cuda_status(e);
-    ProdArgs prod{rstd, static_cast<const uint16_t *>(gamma), y != nullptr};
+    ProdArgs prod{};
+    prod.rstd = rstd;
+    prod.gamma = static_cast<const uint16_t *>(gamma);
+    prod.write_y = y != nullptr;
     return cuda_status(launch_quantize_rmsnorm(a, tm_x, tm_q, tm_qt, tm_y, prod, s));
 }
 

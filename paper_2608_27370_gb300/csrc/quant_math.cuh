@@ -63,6 +63,28 @@ PURO_DEV uint32_t cvt_f32x2(uint64_t v) {
     return cvt_pair<FMT>(lo, hi);
 }
 
+// Codes of two packed pairs as four bytes, ab's low value in the low byte
+// (one move joins the conversions' halves).
+template <int FMT>
+PURO_DEV uint32_t cvt_f32x4(uint64_t ab, uint64_t cd) {
+    uint32_t r;
+    if constexpr (FMT == 0)
+        asm("{\n\t.reg .f32 a, b, c, d;\n\t.reg .b16 lo, hi;\n\t"
+            "mov.b64 {a, b}, %1;\n\tmov.b64 {c, d}, %2;\n\t"
+            "cvt.rn.satfinite.e4m3x2.f32 lo, b, a;\n\tcvt.rn.satfinite.e4m3x2.f32 hi, d, c;\n\t"
+            "mov.b32 %0, {lo, hi};\n\t}"
+            : "=r"(r)
+            : "l"(ab), "l"(cd));
+    else
+        asm("{\n\t.reg .f32 a, b, c, d;\n\t.reg .b16 lo, hi;\n\t"
+            "mov.b64 {a, b}, %1;\n\tmov.b64 {c, d}, %2;\n\t"
+            "cvt.rn.satfinite.e5m2x2.f32 lo, b, a;\n\tcvt.rn.satfinite.e5m2x2.f32 hi, d, c;\n\t"
+            "mov.b32 %0, {lo, hi};\n\t}"
+            : "=r"(r)
+            : "l"(ab), "l"(cd));
+    return r;
+}
+
 // Codes of four values a, b, c, d (exact fp32 widenings of bf16) as four
 // bytes, a in the low byte.  `mul2` holds the multiplier twice: the exact
 // power of two 2^(127-g) (BLOCK) or the fp32 tensor scale (TENSOR).  A
@@ -74,7 +96,7 @@ PURO_DEV uint32_t quant4(float a, float b, float c, float d, uint64_t mul2, bool
                            (((__float_as_uint(c) >> 24) & 0x80u) << 16) | (((__float_as_uint(d) >> 24) & 0x80u) << 24);
         return s | 0x7F7F7F7Fu;
     }
-    return cvt_f32x2<FMT>(mul_f32x2(f32x2(a, b), mul2)) | (cvt_f32x2<FMT>(mul_f32x2(f32x2(c, d), mul2)) << 16);
+    return cvt_f32x4<FMT>(mul_f32x2(f32x2(a, b), mul2), mul_f32x2(f32x2(c, d), mul2));
 }
 
 // Exact 2^(127 - g) as fp32 for g in [0, 247] (always a normal number).

@@ -90,3 +90,22 @@ def test_unfused_rmsnorm_matches_the_fused_one():
     torch.cuda.synchronize()
     assert torch.equal(r1, r2)
     assert torch.equal(y1.view(torch.int16), y2.view(torch.int16))
+
+
+@pytest.mark.parametrize("write_y", [False, True])
+def test_fused_rmsnorm_with_an_unaligned_rstd(write_y):
+    """rstd need only be 4-byte aligned: the same bytes as with an aligned one."""
+    rows, cols = 384, 640
+    h = _h(rows, cols, 951)
+    gamma = W.normal_f32((cols,), 0.1, DEV, 952).add_(1.0).to(torch.bfloat16)
+    got = []
+    for shift in (0, 1, 3):
+        rstd = torch.empty(rows + 4, dtype=torch.float32, device=DEV)[shift:shift + rows]
+        y = torch.zeros((rows, cols), dtype=torch.bfloat16, device=DEV)
+        q = _empty_q(rows, cols)
+        P.puro_fp8_quantize_rmsnorm(h, gamma, 1e-6, P.E4M3, rstd, y if write_y else None, q.rowwise.data,
+                                    q.rowwise.scale, q.colwise.data, q.colwise.scale)
+        torch.cuda.synchronize()
+        got.append([rstd, y.view(torch.int16), q.rowwise.data, q.rowwise.scale, q.colwise.data, q.colwise.scale])
+    for other in got[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(got[0], other))
