@@ -4,9 +4,11 @@ Python binding of ``libpuro_fp8.so`` (C ABI in ``include/puro_fp8.h``).
 Every function here is argument marshalling only: it checks that the torch
 tensors it is handed are CUDA, contiguous and of the right dtype, and passes
 their device pointers, the sizes and the current CUDA stream to the library
-entry point of the same name.  All arithmetic runs in the library's CUDA
-kernels.  There is no fallback: if the library is missing, every call raises
-:class:`PuroError`.
+entry point of the same name.  The calls of a training step do this in native
+code (``csrc/binding.cpp``) for ordinary arguments; anything else it hands
+back, and the ctypes path below it checks the arguments one by one.  All
+arithmetic runs in the library's CUDA kernels.  There is no fallback: if the
+library is missing, every call raises.
 
 The method (paper section "FP8 Mixed-Precision Training"; appendix
 "Production Training Details", paragraph "FP8 implementation pipeline"):
@@ -18,6 +20,8 @@ BF16 output.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from dataclasses import dataclass
 from typing import Optional
@@ -119,6 +123,25 @@ def load_library(path: Optional[str] = None):
     return lib
 
 
+_native = None
+
+
+def _load_native():
+    """The native marshalling module, built and linked against the library at LIB_PATH."""
+    global _native
+    load_library()
+    if not os.path.exists(_build.NATIVE):
+        raise RuntimeError(f"{_build.NATIVE} not found: build it with "
+                           "`python -c 'import __graft_entry__ as g; g.build()'`")
+    name = __name__ + "._native"
+    loader = importlib.machinery.ExtensionFileLoader(name, _build.NATIVE)
+    module = importlib.util.module_from_spec(importlib.util.spec_from_loader(name, loader))
+    loader.exec_module(module)
+    module.set_operand_type(FP8Operand)
+    _native = module
+    return module
+
+
 def _check(fn: str, status: int) -> None:
     if status != PURO_OK:
         raise PuroError(fn, status)
@@ -150,6 +173,9 @@ def _ptr(t: Optional[torch.Tensor], dtype=None, name: str = "tensor") -> Optiona
 # Entry points (same names as the C ABI)
 # --------------------------------------------------------------------------
 def puro_fp8_amax(x: torch.Tensor, amax_bits: torch.Tensor, stream=None) -> None:
+    st = (_native or _load_native()).puro_fp8_amax(x, amax_bits, stream)
+    if st is not None:
+        return _check("puro_fp8_amax", st)
     rows, cols = (x.shape[0], x.shape[1]) if x.dim() == 2 else (1, x.numel())
     st = load_library().puro_fp8_amax(_ptr(x, torch.bfloat16, "x"), rows, cols,
                                       _ptr(amax_bits, (torch.int32, torch.uint32), "amax_bits"), _stream(stream))
@@ -160,6 +186,10 @@ def puro_fp8_quantize(x: torch.Tensor, fmt: int, scaling: int, role: int, amax_b
                       q: torch.Tensor, scale: torch.Tensor, q_t: Optional[torch.Tensor] = None,
                       scale_t: Optional[torch.Tensor] = None, dev_status: Optional[torch.Tensor] = None,
                       stream=None) -> None:
+    st = (_native or _load_native()).puro_fp8_quantize(x, fmt, scaling, role, amax_bits, q, scale, q_t,
+                                                    scale_t, dev_status, stream)
+    if st is not None:
+        return _check("puro_fp8_quantize", st)
     rows, cols = x.shape
     u8 = torch.uint8
     sdt = u8 if scaling == SCALE_BLOCK else torch.float32
@@ -178,6 +208,10 @@ def puro_fp8_quantize_rmsnorm(h: torch.Tensor, gamma: Optional[torch.Tensor], ep
     """RMSNorm of the rows of h (bf16, optional bf16 gain) fused ahead of the
     blockwise activation quantiser: writes rstd (fp32 [rows]), optionally y
     (bf16), and the codes and scales as puro_fp8_quantize does."""
+    st = (_native or _load_native()).puro_fp8_quantize_rmsnorm(h, gamma, eps, fmt, rstd, y, q, scale, q_t,
+                                                            scale_t, dev_status, stream)
+    if st is not None:
+        return _check("puro_fp8_quantize_rmsnorm", st)
     rows, cols = h.shape
     u8 = torch.uint8
     st = load_library().puro_fp8_quantize_rmsnorm(
@@ -234,6 +268,10 @@ def puro_fp8_quantize_weights(entries, fmt: int = E4M3, dev_status: Optional[tor
     of (w, Quantized) pairs or a table from weight_table().  Same bytes as
     quantize(w, fmt, SCALE_BLOCK, ROLE_WEIGHT, out=q) for each."""
     table = entries if isinstance(entries, ctypes.Array) else weight_table(entries)
+    st = (_native or _load_native()).puro_fp8_quantize_weights(ctypes.addressof(table), table.count, fmt, dev_status,
+                                                               stream)
+    if st is not None:
+        return _check("puro_fp8_quantize_weights", st)
     st = load_library().puro_fp8_quantize_weights(table, table.count, fmt,
                                                   _ptr(dev_status, torch.int32, "dev_status"), _stream(stream))
     _check("puro_fp8_quantize_weights", st)
@@ -246,6 +284,10 @@ def puro_fp8_quantize_swiglu(gate: torch.Tensor, up: torch.Tensor, fmt: int, y: 
     """SwiGLU (silu(gate) * up, bf16) fused ahead of the blockwise activation
     quantiser: writes the codes and scales as puro_fp8_quantize does, and y
     (bf16) only when given.  gate and up may be row-strided views."""
+    st = (_native or _load_native()).puro_fp8_quantize_swiglu(gate, up, fmt, y, q, scale, q_t, scale_t,
+                                                           dev_status, stream)
+    if st is not None:
+        return _check("puro_fp8_quantize_swiglu", st)
     g, u, rows, cols, ld = _gate_up(gate, up)
     u8 = torch.uint8
     st = load_library().puro_fp8_quantize_swiglu(
@@ -373,6 +415,9 @@ class FP8Operand:
 
 def _gemm(name: str, a: FP8Operand, b: FP8Operand, out: torch.Tensor, workspace, dev_status, stream,
           out_dtype=torch.bfloat16) -> None:
+    st = getattr(_native or _load_native(), name)(a, b, out, workspace, dev_status, stream)
+    if st is not None:
+        return _check(name, st)
     ca, cb = a.as_c(), b.as_c()
     ws_ptr = _ptr(workspace, None, "workspace")
     ws_bytes = workspace.numel() * workspace.element_size() if workspace is not None else 0
@@ -398,6 +443,10 @@ def puro_fp8_linear_backward(dy: FP8Operand, w_t: FP8Operand, dx: torch.Tensor, 
                              x_t: FP8Operand, dw: torch.Tensor, workspace=None, dev_status=None, stream=None) -> None:
     """dX [M,K] = dY . W and dW [N,K] = dY^T . X in one call (one grouped
     launch when both are unsplit block-scaled GEMMs)."""
+    st = (_native or _load_native()).puro_fp8_linear_backward(dy, w_t, dx, dy_t, x_t, dw, workspace,
+                                                           dev_status, stream)
+    if st is not None:
+        return _check("puro_fp8_linear_backward", st)
     c = [op.as_c() for op in (dy, w_t, dy_t, x_t)]
     ws_bytes = workspace.numel() * workspace.element_size() if workspace is not None else 0
     st = load_library().puro_fp8_linear_backward(
@@ -414,6 +463,10 @@ def puro_fp8_linear_dgrad_quantize(dy: FP8Operand, w_t: FP8Operand, fmt: int, dx
     GEMM's epilogue into the blockwise activation copies (dxq [M,K] with
     1x128 groups; dxq_t [K,M] with 128-row groups, optional); dx (bf16) is
     written only when given."""
+    st = (_native or _load_native()).puro_fp8_linear_dgrad_quantize(dy, w_t, fmt, dx, dxq, dxq_scale, dxq_t,
+                                                                 dxq_t_scale, dev_status, stream)
+    if st is not None:
+        return _check("puro_fp8_linear_dgrad_quantize", st)
     ca, cb = dy.as_c(), w_t.as_c()
     u8 = torch.uint8
     st = load_library().puro_fp8_linear_dgrad_quantize(
@@ -469,6 +522,9 @@ def puro_fp8_get_status(dev_status: torch.Tensor, stream=None) -> int:
 
 
 def _bf16(name, a, b, out, M, N, K, dev_status, stream):
+    st = getattr(_native or _load_native(), name)(a, b, out, M, N, K, dev_status, stream)
+    if st is not None:
+        return _check(name, st)
     fn = getattr(load_library(), name)
     st = fn(_ptr(a, torch.bfloat16, "a"), _ptr(b, torch.bfloat16, "b"), _ptr(out, torch.bfloat16, "out"), M, N, K,
             _ptr(dev_status, torch.int32, "dev_status"), _stream(stream))

@@ -2,7 +2,9 @@
 
 Five translation units are compiled in parallel and linked into one shared
 object with the CUDA runtime linked statically, so the library loads on a
-machine without a GPU driver (only the first CUDA call needs one).
+machine without a GPU driver (only the first CUDA call needs one).  Beside it
+the Python binding's native marshalling module _native.so is compiled against
+the installed torch's headers and linked against the library.
 """
 from __future__ import annotations
 
@@ -10,6 +12,7 @@ import concurrent.futures as cf
 import os
 import shutil
 import subprocess
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -17,6 +20,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libpuro_fp8.so")
+NATIVE = os.path.join(PKG, "_native.so")
+BINDING = os.path.join(CSRC, "binding.cpp")
 SOURCES = ["api.cu", "quantize.cu", "gemm.cu", "noalloc.cu", "muonh.cu"]
 HEADERS = ["ptx.cuh", "internal.h", "quant_math.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -32,10 +37,10 @@ def _nvcc() -> str:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(NATIVE):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS] + [os.path.join(INCLUDE, "puro_fp8.h"),
+    t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
+    deps = [BINDING] + [os.path.join(CSRC, f) for f in SOURCES + HEADERS] + [os.path.join(INCLUDE, "puro_fp8.h"),
                                                                   os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -59,14 +64,44 @@ def build(force: bool = False, verbose: bool = False) -> str:
             print(r.stdout, r.stderr, flush=True)
         return obj
 
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+    def compile_binding() -> str:
+        import torch  # headers only: the module is compiled for the torch it is imported beside
+
+        inc = os.path.join(os.path.dirname(torch.__file__), "include")
+        obj = os.path.join(BUILD, "binding.o")
+        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", "-Wall",
+               "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI, "-isystem", inc, "-isystem",
+               os.path.join(inc, "torch", "csrc", "api", "include"), "-isystem", sysconfig.get_paths()["include"],
+               "-isystem", os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include"),
+               "-I", INCLUDE, "-c", BINDING, "-o", obj]
+        if verbose:
+            print(" ".join(cmd), flush=True)
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            raise RuntimeError(f"g++ failed on binding.cpp:\n{r.stdout}\n{r.stderr}")
+        return obj
+
+    with cf.ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
+        binding = ex.submit(compile_binding)
         objs = list(ex.map(compile_one, SOURCES))
+        binding_obj = binding.result()
     tmp = LIB + ".tmp.%d" % os.getpid()
     cmd = [nvcc, *ARCH, "-shared", "-cudart", "static", "-o", tmp, *objs]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, LIB)
+
+    import torch
+
+    libs = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = NATIVE + ".tmp.%d" % os.getpid()
+    cmd = ["g++", "-shared", "-o", tmp, binding_obj, "-L", PKG, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN",
+           "-L", libs, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"link of the binding failed:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, NATIVE)
     return LIB
 
 

@@ -1,0 +1,158 @@
+"""The native argument marshalling against the general path: it leaves every
+argument that is not of the ordinary kind to the Python code (which raises or
+handles it), and for ordinary arguments both give the same bytes and errors.
+"""
+import ctypes
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2608_27370_gb300 as P
+from paper_2608_27370_gb300 import workloads as W
+
+DEV = "cuda"
+u8, i32, bf16, f32 = torch.uint8, torch.int32, torch.bfloat16, torch.float32
+
+
+class _General:
+    """Stands in for the native module: every call goes to the general path."""
+
+    def __getattr__(self, name):
+        return lambda *a: None
+
+
+def _buffers(dev, M=256, N=384, K=128):
+    e = lambda dt, *s: torch.zeros(s, dtype=dt, device=dev)  # noqa: E731
+    op = lambda r, c, role=P.ROLE_ACT: P.FP8Operand(e(u8, r, c), e(u8, *P.scale_vec_shape(r, c)), role=role)  # noqa: E731
+    b = dict(x=e(bf16, M, K), st=e(i32, 1), ws=e(u8, 64), amax=e(i32, 1), xo=op(M, K), xt=op(K, M), wo=op(N, K),
+             wt=op(K, N), dyo=op(M, N), dyt=op(N, M), y=e(bf16, M, N), dx=e(bf16, M, K), dw=e(bf16, N, K),
+             main=e(f32, N, K), rstd=e(f32, M), gu=e(bf16, M, 2 * K), a=e(bf16, M, K), w=e(bf16, N, K), sf=e(f32, 1))
+    b["dxo"], b["dxt"] = op(M, K), op(K, M)
+    b["table"] = (P.puro_fp8_weight_t * 1)()
+    return b
+
+
+def _native_args(b, M=256, N=384, K=128):
+    """Every native function with a whole set of ordinary arguments."""
+    q = lambda o, t: (o.data, o.scale, t.data, t.scale)  # noqa: E731
+    st = (b["st"], None)
+    return {
+        "puro_fp8_amax": (b["x"], b["amax"], None),
+        "puro_fp8_quantize": (b["x"], 0, 1, 0, None, *q(b["xo"], b["xt"]), *st),
+        "puro_fp8_quantize_rmsnorm": (b["x"], None, 1e-6, 0, b["rstd"], b["a"], *q(b["xo"], b["xt"]), *st),
+        "puro_fp8_quantize_swiglu": (b["gu"][:, :K], b["gu"][:, K:], 0, b["a"], *q(b["xo"], b["xt"]), *st),
+        "puro_fp8_quantize_weights": (ctypes.addressof(b["table"]), 1, 0, *st),
+        "puro_fp8_linear_fprop": (b["xo"], b["wo"], b["y"], b["ws"], *st),
+        "puro_fp8_linear_dgrad": (b["dyo"], b["wt"], b["dx"], b["ws"], *st),
+        "puro_fp8_linear_wgrad": (b["dyt"], b["xt"], b["dw"], b["ws"], *st),
+        "puro_fp8_linear_wgrad_main_grad": (b["dyt"], b["xt"], b["main"], b["ws"], *st),
+        "puro_fp8_linear_backward": (b["dyo"], b["wt"], b["dx"], b["dyt"], b["xt"], b["dw"], b["ws"], *st),
+        "puro_fp8_linear_dgrad_quantize": (b["dyo"], b["wt"], 0, b["dx"], *q(b["dxo"], b["dxt"]), *st),
+        "puro_bf16_linear_fprop": (b["x"], b["w"], b["y"], M, N, K, *st),
+        "puro_bf16_linear_dgrad": (b["y"], b["dw"], b["dx"], M, N, K, *st),
+        "puro_bf16_linear_wgrad": (b["y"], b["x"], b["dw"], M, N, K, *st),
+    }
+
+
+@pytest.mark.parametrize("name", sorted(_native_args(_buffers("cpu"))))
+def test_native_leaves_unusual_arguments_alone(name):
+    native = P._load_native()
+    fn, args = getattr(native, name), list(_native_args(_buffers("cpu"))[name])
+    assert fn() is None and fn(*args, None) is None  # another number of arguments
+    if name != "puro_fp8_quantize_weights":
+        assert fn(*args) is None  # host tensors
+    odd = [object(), "x", 1.5, True, 2 ** 70, np.zeros(4), torch.zeros(0), torch.zeros(4, device="meta"),
+           torch.zeros(4, 4).t(), torch.nested.nested_tensor([torch.zeros(2)])]
+    for k in range(len(args)):
+        for o in odd:
+            if name == "puro_fp8_quantize_weights" and k == 0:
+                continue  # an address is taken as it is
+            assert fn(*args[:k], o, *args[k + 1:]) is None, (k, type(o))
+
+
+def test_native_refuses_other_operand_classes():
+    class Sub(P.FP8Operand):
+        pass
+
+    b = _buffers("cpu")
+    o = Sub(b["xo"].data, b["xo"].scale)
+    assert P._load_native().puro_fp8_linear_fprop(o, b["wo"], b["y"], None, None, None) is None
+
+
+def _random(b):
+    for k, t in enumerate(("x", "w", "gu")):
+        b[t].copy_(W.normal_bf16(tuple(b[t].shape), 1.0, DEV, 40 + k))
+    for k, t in enumerate(("xo", "xt", "wo", "wt", "dyo", "dyt")):
+        r = W.normal_bf16((b[t].rows, b[t].red), 1.0, DEV, 50 + k)
+        P.puro_fp8_quantize(r, 0, 1, 0, None, b[t].data, b[t].scale)
+
+
+def _calls(b, M=256, N=384, K=128):
+    for name, args in _native_args(b, M, N, K).items():
+        if name == "puro_fp8_quantize_weights":
+            q = P.Quantized(b["wo"], P.FP8Operand(b["wt"].data, b["wt"].scale))
+            yield name, lambda q=q: P.puro_fp8_quantize_weights([(b["w"], q)], 0, b["st"])
+        else:
+            yield name, lambda name=name, args=args: getattr(P, name)(*args)
+    yield "stream object", lambda: P.puro_fp8_linear_fprop(b["xo"], b["wo"], b["y"], b["ws"], b["st"],
+                                                           torch.cuda.current_stream())
+    yield "per-tensor", lambda: P.puro_fp8_quantize(b["x"], 1, 0, 0, b["amax"], b["xo"].data, b["sf"], b["xt"].data,
+                                                    None)
+    yield "keywords", lambda: P.puro_fp8_linear_dgrad(b["dyo"], b["wt"], dx=b["dx"], dev_status=b["st"])
+
+
+@pytest.mark.gpu
+def test_both_paths_give_the_same_bytes():
+    P._load_native()
+    got = []
+    native = P._native
+    try:
+        for route in (native, _General()):
+            P._native = route
+            b = _buffers(DEV)
+            _random(b)
+            for name, call in _calls(b):
+                call()
+            torch.cuda.synchronize()
+            flat = []
+            for k in sorted(b):
+                v = b[k]
+                flat += [v.data, v.scale] if isinstance(v, P.FP8Operand) else [v] if torch.is_tensor(v) else []
+            got.append([t.contiguous().view(u8) for t in flat])
+    finally:
+        P._native = native
+    assert all(torch.equal(a, c) for a, c in zip(*got))
+    assert any(int(t.count_nonzero()) for t in got[0])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("route", ["native", "general"])
+def test_errors_are_the_same(route):
+    native = P._load_native()
+    b = _buffers(DEV)
+    q = (b["xo"].data, b["xo"].scale, b["xt"].data, b["xt"].scale)
+    try:
+        P._native = native if route == "native" else _General()
+        with pytest.raises(ValueError, match="x has dtype"):
+            P.puro_fp8_quantize(b["x"].float(), 0, 1, 0, None, *q)
+        with pytest.raises(ValueError, match="x must be contiguous"):
+            P.puro_fp8_quantize(b["gu"][:, :128], 0, 1, 0, None, *q)
+        with pytest.raises(ValueError, match="scale has dtype"):
+            P.puro_fp8_quantize(b["x"], 0, 1, 0, None, q[0], b["sf"], q[2], q[3])
+        with pytest.raises(ValueError, match="out must be a CUDA tensor"):
+            P.puro_fp8_linear_fprop(b["xo"], b["wo"], b["y"].cpu())
+        with pytest.raises(ValueError, match="unit column stride"):
+            P.puro_fp8_quantize_swiglu(b["gu"].t(), b["gu"].t(), 0, None, *q)
+        with pytest.raises(AttributeError):
+            P.puro_fp8_linear_fprop(None, b["wo"], b["y"])
+        for call in (lambda: P.puro_fp8_quantize(b["x"], 7, 1, 0, None, *q),
+                     lambda: P.puro_fp8_linear_fprop(b["xo"], b["dyo"], b["y"]),
+                     lambda: P.puro_fp8_linear_fprop(b["xo"], b["wo"], None),
+                     lambda: P.puro_fp8_linear_fprop(P.FP8Operand(b["xo"].data[:0], b["xo"].scale), b["wo"], b["y"]),
+                     lambda: P.puro_fp8_quantize_rmsnorm(b["x"], None, -1.0, 0, b["rstd"], None, *q)):
+            with pytest.raises(P.PuroError) as e:
+                call()
+            assert e.value.status == P.PURO_ERR_INVALID_ARG
+    finally:
+        P._native = native
