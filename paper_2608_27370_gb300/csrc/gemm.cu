@@ -72,6 +72,7 @@ constexpr int kThreads = 256;
 constexpr int kTmemCols = 512;
 constexpr int kSfColsPerSet = 12;  // 4 for A (128 rows) + 8 for B (up to 256 rows)
 constexpr int kSfSets = 2;         // double-buffered across groups of four k-blocks
+constexpr uint32_t kAllocBarrier = 7, kLeaveBarrier = 8;  // named barriers (the quantising epilogue uses 1..6)
 constexpr int kSfbSlots = 4;       // BN = 224: ring of helper-built B scale images
 constexpr uint64_t kDrainTimeoutNs = 2000000000ull;
 constexpr uint64_t kSettleNs = 200000ull;  // after an abort: let the peer-counted copies land
@@ -171,6 +172,13 @@ template <class Smem>
 PURO_DEV void record_timeout(Smem &sm, int32_t *status) {
     sm.abort_flag = 1;
     if (status) atomicExch(status, kStatusTimeout);
+}
+
+// A wait of the lone issuing thread: the abort flag is read only while the
+// barrier is incomplete (an aborting role stops feeding it).
+template <class Smem>
+PURO_DEV bool wait_unless_aborted(Smem &sm, uint64_t *bar, uint32_t parity, uint64_t wait_ns) {
+    return mbar_try_wait(bar, parity) || (sm.abort_flag == 0 && mbar_wait_bounded(bar, parity, wait_ns));
 }
 
 // One unit of work: a 256 x BN pair tile and a chunk of the reduction.
@@ -516,6 +524,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
     constexpr int kStages = Smem::kStages;
     constexpr bool kMX = (KIND == kGemmFP8Block);
     constexpr bool kHelper = kMX && Smem::kSfbByHelper;
+    constexpr bool OUT_F32 = (OUT == kGemmOutF32Partial || OUT == kGemmOutF32Add);
+    constexpr bool OUT_Q = (OUT == kGemmOutQuant);
+    // The narrow forms run few tiles a launch: the issuing thread waits alone
+    // (a 128-wide stage's eight MMAs take 512 cycles of the tensor pipe and the
+    // waits, copies and commit of a voting warp 420 more; a 256-wide stage takes
+    // 1024 and hides them), and the epilogue arrives at the closing cluster
+    // barrier ahead of its last stores.  On the 256-wide form the former changes
+    // nothing and the latter costs 0.5%.
+    constexpr bool kLeanIssue = BN < 256 && !kHelper;
+    constexpr bool kEarlyLeave = BN < 256 && !OUT_Q;
     constexpr bool kShifted = kMX && BN == 256;         // shared-half accumulators
     constexpr int kAccBufs = kShifted ? 1 : 2;          // hand-off barrier pairs (tfull / tempty)
     constexpr int kAccShift = kShifted ? 128 : 256;     // column offset between consecutive tiles' accumulators
@@ -526,8 +544,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
     constexpr int kKSteps = kAtomBytes / 32;            // MMAs per atom (32 bytes of K each)
     constexpr uint32_t kStageBytes = (kBM + kBNHalf) * kBKBytes;  // one CTA's operand bytes per stage
     constexpr uint32_t kSfBytes = kHelper ? 512u : 512u + 512u * Smem::kSfbChunks;  // one CTA's TMA scale bytes per group
-    constexpr bool OUT_F32 = (OUT == kGemmOutF32Partial || OUT == kGemmOutF32Add);
-    constexpr bool OUT_Q = (OUT == kGemmOutQuant);
     static_assert(BN == 256 || BN == 192 || BN == 128 || (BN == 224 && kMX && OUT == kGemmOutBF16),
                   "the 224-wide form is block-scaled, BF16 out");
     static_assert(OUT != kGemmOutF32Partial || BN == 256, "split reductions run 256-wide");
@@ -573,19 +589,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
             tma_prefetch_desc(&tm_sfa1);
             tma_prefetch_desc(&tm_sfb1);
         }
-
     }
+    if (warp == 0) __syncwarp();
+    cluster_arrive();  // waited for below: both CTAs' barriers exist before any copy or arrival targets them
     if (warp == 1) {
         tmem_alloc_pair(&sm.tmem_base, kTmemCols);
         tmem_relinquish_alloc_permit_pair();
     }
-    tc_fence_before_sync();
-    __syncthreads();
-    cluster_sync();  // both CTAs' barriers exist before any copy or arrival targets them
-    tc_fence_after_sync();
+    // The producer does not use tensor memory: its first copies do not wait for the allocation.
+    if (warp != 0) {
+        tc_fence_before_sync();
+        named_bar_sync(kAllocBarrier, gemm_threads<OUT>() - 32);
+        tc_fence_after_sync();
+    }
+    cluster_wait();
     pdl_wait();  // the set-up above overlaps the previous kernel's tail
     pdl_launch_dependents();
-    const uint32_t tmem = sm.tmem_base;
+    const uint32_t tmem = warp != 0 ? sm.tmem_base : 0u;
+    // Arrive at the closing cluster barrier: this warp is done with tensor
+    // memory and the peer's barriers.
+    bool left = false;
+    auto leave = [&] {
+        tc_fence_before_sync();
+        __syncwarp();
+        cluster_arrive();
+        if (warp >= 4) named_bar_arrive(kLeaveBarrier, gemm_threads<OUT>() - 96);  // lets warp 1 go on
+        left = true;
+    };
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
@@ -656,88 +686,122 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
         }
     } else if (warp == 1 && rank == 0) {
         // ------------------------------------------------ MMA issuer (even CTA)
-        uint32_t stage = 0, phase = 0;
-        uint32_t gseq = 0;  // groups of four k-blocks started (BN = 224: slot of the scale ring)
-        bool aborted = false;
-        int local = 0;
-        PairUnits units(p, pair, num_pairs);
-        for (int u = units.next(); u >= 0 && !aborted; u = units.next(), ++local) {
-            const WorkUnit wu = work_unit<BN>(p, u);
-            const int buf = local % kAccBufs;
-            const uint32_t acc_phase = static_cast<uint32_t>(local / kAccBufs) & 1u;
-            bool ok = (sm.abort_flag == 0) && mbar_wait_bounded(&sm.tempty[buf], acc_phase ^ 1u, p.wait_ns);
-            if (!__all_sync(0xFFFFFFFFu, ok)) {
-                if (lane == 0) record_timeout(sm, p.status);
-                aborted = true;
-                break;
-            }
-            tc_fence_after_sync();
-            const uint32_t d_tmem = tmem + static_cast<uint32_t>((local & 1) * kAccShift);
+        // One stage's scale copies, MMAs and release, by one thread.
+        auto issue_stage = [&](const WorkUnit &wu, int kb, uint32_t stage, uint32_t slot, uint32_t d_tmem) {
+            const bool group_start = kMX && (kb % kStagesPerGroup) == 0;
+            const uint32_t sfa_col = kSfBase + ((kb / kStagesPerGroup) & 1) * kSfColsPerSet;
+            const uint32_t sfb_col = sfa_col + 4;
             // a 192-wide tile starts at row 0 or 64 of its first 128-row scale chunk: 32 rows per column
             const uint32_t sfb_shift = BN == 192 ? static_cast<uint32_t>(wu.n0 % 128) / 32u : 0u;
-
-            for (int kb = wu.kb0; kb < wu.kb1; ++kb) {
-                const bool group_start = kMX && (kb % kStagesPerGroup) == 0;
-                const uint32_t slot = gseq % kSfbSlots;
-                ok = (sm.abort_flag == 0) && mbar_wait_bounded(&sm.full[stage], phase, p.wait_ns);
-                if (kHelper && group_start)
-                    ok = ok && mbar_wait_bounded(&sm.sfb_full[slot], (gseq / kSfbSlots) & 1u, p.wait_ns);
+            if constexpr (kMX) {
+                if (group_start) {  // new group of four k-blocks: its scale vectors
+                    const uint8_t *sfb_src = kHelper ? sm.sf_b[slot] : sm.sf_b[stage];
+                    tmem_cp_pair_32x128b_warpx4(tmem + sfa_col, smem_desc_plain_16B_rows(smem_u32(sm.sf_a[stage])));
+                    tmem_cp_pair_32x128b_warpx4(tmem + sfb_col, smem_desc_plain_16B_rows(smem_u32(sfb_src)));
+                    if constexpr (Smem::kSfbChunks == 2)
+                        tmem_cp_pair_32x128b_warpx4(tmem + sfb_col + 4,
+                                                    smem_desc_plain_16B_rows(smem_u32(sfb_src + 512)));
+                }
+            }
+#pragma unroll
+            for (int at = 0; at < kAtoms; ++at) {
+                uint32_t idesc = wu.problem ? p.idesc1 : p.idesc;
+                if constexpr (kMX) {
+                    const uint32_t sf_id = static_cast<uint32_t>((kb * kAtoms + at) & 3);  // k-block in its group
+                    idesc |= (sf_id << 29) | (sf_id << 4);
+                }
+                const uint32_t a_addr = smem_u32(sm.a[stage][at]);
+                const uint32_t b_addr = smem_u32(sm.b[stage][at]);
+#pragma unroll
+                for (int k = 0; k < kKSteps; ++k) {
+                    const uint64_t ad = smem_desc_k_sw128(a_addr + 32 * k);
+                    const uint64_t bd = smem_desc_k_sw128(b_addr + 32 * k);
+                    const uint32_t acc = (kb > wu.kb0 || at > 0 || k > 0) ? 1u : 0u;
+                    if constexpr (KIND == kGemmBF16)
+                        mma_pair_f16(d_tmem, ad, bd, idesc, acc);
+                    else if constexpr (KIND == kGemmFP8Tensor)
+                        mma_pair_f8(d_tmem, ad, bd, idesc, acc);
+                    else
+                        mma_pair_mxf8(d_tmem, ad, bd, idesc, tmem + sfa_col, tmem + sfb_col + sfb_shift, acc);
+                }
+            }
+            tc_commit_pair_multicast(&sm.empty[stage], 0x3);  // stage reusable in both CTAs
+            // the scale image is free once its copies (issued above) are done
+            if (kHelper && group_start) tc_commit_pair_multicast(&sm.sfb_empty[slot], 0x3);
+        };
+        uint32_t stage = 0, phase = 0;
+        if constexpr (kLeanIssue) {
+            if (lane == 0) {
+                bool aborted = false;
+                int local = 0;
+                PairUnits units(p, pair, num_pairs);
+                for (int u = units.next(); u >= 0 && !aborted; u = units.next(), ++local) {
+                    const WorkUnit wu = work_unit<BN>(p, u);
+                    const int buf = local % kAccBufs;
+                    const uint32_t acc_phase = static_cast<uint32_t>(local / kAccBufs) & 1u;
+                    aborted = !wait_unless_aborted(sm, &sm.tempty[buf], acc_phase ^ 1u, p.wait_ns);
+                    const uint32_t d_tmem = tmem + static_cast<uint32_t>((local & 1) * kAccShift);
+                    for (int kb = wu.kb0; kb < wu.kb1 && !aborted; ++kb) {
+                        if (!wait_unless_aborted(sm, &sm.full[stage], phase, p.wait_ns)) {
+                            aborted = true;
+                            break;
+                        }
+                        tc_fence_after_sync();
+                        issue_stage(wu, kb, stage, 0, d_tmem);
+                        if (++stage == kStages) {
+                            stage = 0;
+                            phase ^= 1u;
+                        }
+                    }
+                    if (aborted) {
+                        record_timeout(sm, p.status);
+                        break;
+                    }
+                    tc_commit_pair_multicast(&sm.tfull[buf], 0x3);  // accumulator complete in both CTAs
+                }
+            }
+            __syncwarp();
+        } else {
+            uint32_t gseq = 0;  // groups of four k-blocks started (BN = 224: slot of the scale ring)
+            bool aborted = false;
+            int local = 0;
+            PairUnits units(p, pair, num_pairs);
+            for (int u = units.next(); u >= 0 && !aborted; u = units.next(), ++local) {
+                const WorkUnit wu = work_unit<BN>(p, u);
+                const int buf = local % kAccBufs;
+                const uint32_t acc_phase = static_cast<uint32_t>(local / kAccBufs) & 1u;
+                bool ok = (sm.abort_flag == 0) && mbar_wait_bounded(&sm.tempty[buf], acc_phase ^ 1u, p.wait_ns);
                 if (!__all_sync(0xFFFFFFFFu, ok)) {
                     if (lane == 0) record_timeout(sm, p.status);
                     aborted = true;
                     break;
                 }
                 tc_fence_after_sync();
-                if (lane == 0) {
-                    const uint32_t sfa_col = kSfBase + ((kb / kStagesPerGroup) & 1) * kSfColsPerSet;
-                    const uint32_t sfb_col = sfa_col + 4;
-                    if constexpr (kMX) {
-                        if (group_start) {  // new group of four k-blocks: its scale vectors
-                            const uint8_t *sfb_src = kHelper ? sm.sf_b[slot] : sm.sf_b[stage];
-                            tmem_cp_pair_32x128b_warpx4(tmem + sfa_col,
-                                                        smem_desc_plain_16B_rows(smem_u32(sm.sf_a[stage])));
-                            tmem_cp_pair_32x128b_warpx4(tmem + sfb_col, smem_desc_plain_16B_rows(smem_u32(sfb_src)));
-                            if constexpr (Smem::kSfbChunks == 2)
-                                tmem_cp_pair_32x128b_warpx4(tmem + sfb_col + 4,
-                                                            smem_desc_plain_16B_rows(smem_u32(sfb_src + 512)));
-                        }
+                const uint32_t d_tmem = tmem + static_cast<uint32_t>((local & 1) * kAccShift);
+                for (int kb = wu.kb0; kb < wu.kb1; ++kb) {
+                    const bool group_start = kMX && (kb % kStagesPerGroup) == 0;
+                    const uint32_t slot = gseq % kSfbSlots;
+                    ok = (sm.abort_flag == 0) && mbar_wait_bounded(&sm.full[stage], phase, p.wait_ns);
+                    if (kHelper && group_start)
+                        ok = ok && mbar_wait_bounded(&sm.sfb_full[slot], (gseq / kSfbSlots) & 1u, p.wait_ns);
+                    if (!__all_sync(0xFFFFFFFFu, ok)) {
+                        if (lane == 0) record_timeout(sm, p.status);
+                        aborted = true;
+                        break;
                     }
-#pragma unroll
-                    for (int at = 0; at < kAtoms; ++at) {
-                        uint32_t idesc = wu.problem ? p.idesc1 : p.idesc;
-                        if constexpr (kMX) {
-                            const uint32_t sf_id = static_cast<uint32_t>((kb * kAtoms + at) & 3);  // k-block in its group
-                            idesc |= (sf_id << 29) | (sf_id << 4);
-                        }
-                        const uint32_t a_addr = smem_u32(sm.a[stage][at]);
-                        const uint32_t b_addr = smem_u32(sm.b[stage][at]);
-#pragma unroll
-                        for (int k = 0; k < kKSteps; ++k) {
-                            const uint64_t ad = smem_desc_k_sw128(a_addr + 32 * k);
-                            const uint64_t bd = smem_desc_k_sw128(b_addr + 32 * k);
-                            const uint32_t acc = (kb > wu.kb0 || at > 0 || k > 0) ? 1u : 0u;
-                            if constexpr (KIND == kGemmBF16)
-                                mma_pair_f16(d_tmem, ad, bd, idesc, acc);
-                            else if constexpr (KIND == kGemmFP8Tensor)
-                                mma_pair_f8(d_tmem, ad, bd, idesc, acc);
-                            else
-                                mma_pair_mxf8(d_tmem, ad, bd, idesc, tmem + sfa_col, tmem + sfb_col + sfb_shift, acc);
-                        }
+                    tc_fence_after_sync();
+                    if (lane == 0) issue_stage(wu, kb, stage, slot, d_tmem);
+                    __syncwarp();
+                    if (group_start) ++gseq;
+                    if (++stage == kStages) {
+                        stage = 0;
+                        phase ^= 1u;
                     }
-                    tc_commit_pair_multicast(&sm.empty[stage], 0x3);  // stage reusable in both CTAs
-                    // the scale image is free once its copies (issued above) are done
-                    if (kHelper && group_start) tc_commit_pair_multicast(&sm.sfb_empty[slot], 0x3);
                 }
+                if (aborted) break;
+                if (lane == 0) tc_commit_pair_multicast(&sm.tfull[buf], 0x3);  // accumulator complete in both CTAs
                 __syncwarp();
-                if (group_start) ++gseq;
-                if (++stage == kStages) {
-                    stage = 0;
-                    phase ^= 1u;
-                }
             }
-            if (aborted) break;
-            if (lane == 0) tc_commit_pair_multicast(&sm.tfull[buf], 0x3);  // accumulator complete in both CTAs
-            __syncwarp();
         }
         // All MMAs and copies issued by this warp complete before teardown.
         if (lane == 0) {
@@ -811,7 +875,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
         int local = 0;
         uint32_t pieces = 0;  // BF16 output: 32-column pieces stored, alternating staging halves
         PairUnits units(p, pair, num_pairs);
-        for (int u = units.next(); u >= 0; u = units.next(), ++local) {
+        for (int u = units.next(), un = 0; u >= 0; u = kEarlyLeave ? un : units.next(), ++local) {
+            if constexpr (kEarlyLeave) un = units.next();
             const WorkUnit wu = work_unit<BN>(p, u);
             const int m0 = wu.m0 + kBM * static_cast<int>(rank), n0 = wu.n0;  // this CTA's rows
             const int buf = local % kAccBufs;
@@ -859,6 +924,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                         __syncwarp();
                         if (lane == 0) mbar_arrive_cluster_cta_scope(tempty0 + 8u * buf);  // accumulator free for the next tile
                     }
+                    if (kEarlyLeave && hh == kHalves - 1 && un < 0) leave();  // the last tile is in registers
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
                         const int col = n0 + 128 * h + 32 * c;
@@ -908,6 +974,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                         __syncwarp();
                         if (lane == 0) mbar_arrive_cluster_cta_scope(tempty0 + 8u * buf);  // accumulator free for the next tile
                     }
+                    if (kEarlyLeave && hh == kHalves - 1 && un < 0) leave();  // the last tile is in registers
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
                         const int col = n0 + 128 * h + 32 * c;
@@ -937,11 +1004,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
         __syncwarp();
     }
 
-    tc_fence_before_sync();
+    // The pair's MMAs into both CTAs' tensor memory are complete and read
+    // before it is freed, and no arrival targets a CTA that has left.  The
+    // narrow forms' epilogue warps arrive before their last tile's stores, so
+    // the cluster barrier and the release of tensor memory pass behind those.
+    // Waiting on a cluster barrier takes issue slots, so warps that are done
+    // early wait at the CTA's barriers.
+    if (!left) leave();
+    if (warp == 1) {
+        named_bar_sync(kLeaveBarrier, gemm_threads<OUT>() - 96);  // this CTA's epilogue warps have arrived
+        cluster_wait();
+        tc_fence_after_sync();
+        tmem_dealloc_pair(tmem, kTmemCols);
+    }
     __syncthreads();
-    cluster_sync();  // the pair's MMAs into both CTAs' tensor memory are complete
-    tc_fence_after_sync();
-    if (warp == 1) tmem_dealloc_pair(tmem, kTmemCols);
+    if (warp != 1) cluster_wait();
 }
 
 // Split-K reduction: out[i] = bf16(sum_s ws[s][i]) in fixed order s = 0, 1, ...

@@ -43,6 +43,10 @@ PURO_DEV void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_depe
 PURO_DEV void named_bar_sync(uint32_t id, uint32_t threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
+// Arrive without waiting (others wait with named_bar_sync).
+PURO_DEV void named_bar_arrive(uint32_t id, uint32_t threads) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
 PURO_DEV bool named_bar_and(uint32_t id, uint32_t threads, bool pred) {
     uint32_t r;
     asm volatile(
@@ -199,6 +203,10 @@ PURO_DEV uint32_t cluster_ctarank() {
 PURO_DEV void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+
+// The two halves of cluster_sync, for work in between.
+PURO_DEV void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+PURO_DEV void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // Address of the same shared-memory variable in cluster CTA `rank`.
 PURO_DEV uint32_t mapa_shared(uint32_t saddr, uint32_t rank) {
