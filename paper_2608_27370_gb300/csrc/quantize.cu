@@ -551,6 +551,15 @@ __global__ void __launch_bounds__(kQThreads, 2)
 // entry points require multiples of 128).
 constexpr int kQAThreads = 512;
 
+// max(|a|, |b|) of two bf16 pairs, the signs left as they fall; NaN if either
+// is.  Off the integer pipe, which RMSNorm's widening loads (68.2 -> 67.1 us on
+// [32768, 1536]; no gain without a producer or behind SwiGLU).
+PURO_DEV uint32_t absmax_bf16x2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("max.NaN.xorsign.abs.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
 struct QuantActSmem {
     alignas(1024) uint8_t q_stage[kQT * kQT];    // rowwise codes, plain rows
     alignas(1024) uint8_t qt_stage[kQT * kQT];   // transposed codes, 128B-swizzled rows
@@ -559,6 +568,8 @@ struct QuantActSmem {
     alignas(16) float col_mul[kQT];
     alignas(16) uint8_t row_g[kQT];
     alignas(16) uint8_t col_g[kQT];
+    alignas(16) float rstd[2][kQT];              // kProdRmsNorm: of the tile's rows, with the tile (full[])
+    alignas(16) uint16_t gamma[2][kQT];          // kProdRmsNorm: of the tile's columns
     uint64_t full[2];
 };
 
@@ -596,10 +607,10 @@ PURO_DEV uint2 swiglu_chunk4(uint2 g, uint2 u) {
 // Behind a producer the kernel is bound by its instructions between the tile's
 // three barriers, not by HBM, so the produced block stays in registers (it is
 // written back to shared memory only for a y output), RMSNorm's products are
-// packed in pairs and its rstd and gains are fetched while the tile is waited
-// for.  With the block written back and read again, one product an instruction
-// and a load per row: RMSNorm (both kernels) 72.1 -> 68.8 us on [32768, 1536],
-// 9.7 -> 8.8 on [2048, 2048]; SwiGLU 64.1 -> 62.1 us on [8192, 6144] (4.9 TB/s).
+// packed in pairs and its rstd and gains arrive with the tile.  With the block
+// written back and read again, one product an instruction and a load per row:
+// RMSNorm (both kernels) 71.5 -> 67.0 us on [32768, 1536], 9.6 -> 8.5 on
+// [2048, 2048]; SwiGLU 64.1 -> 62.0 us on [8192, 6144] (4.9 TB/s).
 // Without a producer the plain quantiser runs at 5.8-6.3 TB/s and re-reads the
 // block from shared memory (holding it instead was 1.6% slower on
 // [32768, 17920], 2-3% faster below [8192, 2048]).
@@ -624,9 +635,19 @@ __global__ void __launch_bounds__(kQAThreads, 2)
         if (HAS_T) tma_prefetch_desc(&tm_qt);
     }
     __syncthreads();
-    auto issue_load = [&](const TileWalk &t, int b) {
-        mbar_arrive_expect_tx(&sm.full[b], kQT * kQT * 2);
+    // RMSNorm: the tile's rstd (when 16-byte aligned, which the caller's need
+    // not be) and gains arrive with it, so no thread waits for them.
+    const bool rstd16 = PROD == kProdRmsNorm && (reinterpret_cast<uintptr_t>(prod.rstd) & 15u) == 0;
+    const uint32_t tile_bytes = kQT * kQT * 2 + (rstd16 ? kQT * 4 : 0) + (prod.gamma ? kQT * 2 : 0);
+    auto issue_tile = [&](const TileWalk &t, int b) {
+        mbar_arrive_expect_tx(&sm.full[b], PROD == kProdRmsNorm ? tile_bytes : kQT * kQT * 2);
         tma_load_2d(sm.in[b], &tm_x, &sm.full[b], t.c * kQT, t.r * kQT);
+    };
+    auto issue_vectors = [&](const TileWalk &t, int b) {
+        if constexpr (PROD == kProdRmsNorm) {
+            if (rstd16) bulk_load(sm.rstd[b], prod.rstd + static_cast<int64_t>(t.r) * kQT, kQT * 4, &sm.full[b]);
+            if (prod.gamma) bulk_load(sm.gamma[b], prod.gamma + static_cast<int64_t>(t.c) * kQT, kQT * 2, &sm.full[b]);
+        }
     };
     int tile = blockIdx.x;
     const int step = gridDim.x;
@@ -636,12 +657,15 @@ __global__ void __launch_bounds__(kQAThreads, 2)
     // the same h, whose CTAs all passed their own pdl_wait before this grid
     // could start, so h is complete: the first tile streams in during the
     // rstd pass's tail.  rstd is read behind the wait.
-    if (PROD == kProdRmsNorm && tid == 0 && tile < ntiles) issue_load(cur, 0);
+    if (PROD == kProdRmsNorm && tid == 0 && tile < ntiles) issue_tile(cur, 0);
     bool gave_up = false;  // a zero wait bound is one test right after the load is issued
     if (PROD == kProdRmsNorm && tid == 0 && wait_ns == 0 && tile < ntiles) gave_up = !mbar_test_wait(&sm.full[0], 0);
     pdl_wait();
     pdl_launch_dependents();
-    if (PROD != kProdRmsNorm && tid == 0 && tile < ntiles) issue_load(cur, 0);
+    if (tid == 0 && tile < ntiles) {
+        if (PROD != kProdRmsNorm) issue_tile(cur, 0);
+        issue_vectors(cur, 0);
+    }
     uint2 un[8];  // kProdSwiGlu: this thread's block of u for the current tile
     auto load_up = [&](const TileWalk &t) {
         const int64_t row0 = static_cast<int64_t>(t.r) * kQT + 8 * br;
@@ -657,29 +681,15 @@ __global__ void __launch_bounds__(kQAThreads, 2)
         const int buf = it & 1;
         const int64_t r0 = static_cast<int64_t>(cur.r) * kQT;
         const int64_t c0 = static_cast<int64_t>(cur.c) * kQT;
-        uint64_t gm[2] = {0, 0};  // kProdRmsNorm: the gains of the thread's columns and its rows' rstd,
-        float rs[8];              // fetched while the tile is waited for
-        if constexpr (PROD == kProdRmsNorm) {
-            const float *rp = prod.rstd + r0 + 8 * br;
-            if ((reinterpret_cast<uintptr_t>(rp) & 15u) == 0) {  // the caller's rstd need only be 4-byte aligned
-                const float4 a = *reinterpret_cast<const float4 *>(rp), b = *reinterpret_cast<const float4 *>(rp + 4);
-                rs[0] = a.x, rs[1] = a.y, rs[2] = a.z, rs[3] = a.w, rs[4] = b.x, rs[5] = b.y, rs[6] = b.z, rs[7] = b.w;
-            } else {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) rs[i] = rp[i];
-            }
-            if (prod.gamma) {
-                const uint2 g = __ldg(reinterpret_cast<const uint2 *>(prod.gamma + c0 + 4 * bc));
-                gm[0] = f32x2(bf16_lo(g.x), bf16_hi(g.x));
-                gm[1] = f32x2(bf16_lo(g.y), bf16_hi(g.y));
-            }
-        }
         if (tid == 0) {
             const int next = tile + step;
             // with a y output, the buffer's last reader was the y store of
             // tile it-1: all but the newest bulk group (its code stores) done
             if (PROD != kProdNone && prod.write_y) bulk_wait_group_read<1>();
-            if (next < ntiles) issue_load(nxt, buf ^ 1);  // its buffer was last read before (S4) of it-1
+            if (next < ntiles) {  // its buffer was last read before (S4) of it-1
+                issue_tile(nxt, buf ^ 1);
+                issue_vectors(nxt, buf ^ 1);
+            }
         }
         // Every thread waits on the tile's barrier itself (which makes the
         // TMA-written tile visible to it); the shared buffers written before
@@ -692,6 +702,21 @@ __global__ void __launch_bounds__(kQAThreads, 2)
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[i] = *reinterpret_cast<const uint2 *>(in + (8 * br + i) * kQT + 4 * bc);
         if constexpr (PROD == kProdRmsNorm) {
+            uint64_t gm[2] = {0, 0};
+            if (prod.gamma) {
+                const uint2 g = *reinterpret_cast<const uint2 *>(&sm.gamma[buf][4 * bc]);
+                gm[0] = f32x2(bf16_lo(g.x), bf16_hi(g.x));
+                gm[1] = f32x2(bf16_lo(g.y), bf16_hi(g.y));
+            }
+            float rs[8];
+            if (rstd16) {
+                const float4 a = *reinterpret_cast<const float4 *>(&sm.rstd[buf][8 * br]);
+                const float4 b = *reinterpret_cast<const float4 *>(&sm.rstd[buf][8 * br + 4]);
+                rs[0] = a.x, rs[1] = a.y, rs[2] = a.z, rs[3] = a.w, rs[4] = b.x, rs[5] = b.y, rs[6] = b.z, rs[7] = b.w;
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) rs[i] = prod.rstd[r0 + 8 * br + i];
+            }
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 v[i] = rmsnorm_chunk4(v[i], f32x2(rs[i], rs[i]), gm, prod.gamma != nullptr);
@@ -716,8 +741,13 @@ __global__ void __launch_bounds__(kQAThreads, 2)
             uint32_t rmax[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const uint32_t m = __vmaxu2(v[i].x & 0x7FFF7FFFu, v[i].y & 0x7FFF7FFFu);
-                rmax[i] = __reduce_max_sync(0xFFFFFFFFu, __vmaxu2(m, __byte_perm(m, 0u, 0x1032)));
+                if constexpr (PROD == kProdRmsNorm) {
+                    const uint32_t m = absmax_bf16x2(v[i].x, v[i].y);
+                    rmax[i] = __reduce_max_sync(0xFFFFFFFFu, absmax_bf16x2(m, __byte_perm(m, 0u, 0x1032)) & 0x7FFF7FFFu);
+                } else {
+                    const uint32_t m = __vmaxu2(v[i].x & 0x7FFF7FFFu, v[i].y & 0x7FFF7FFFu);
+                    rmax[i] = __reduce_max_sync(0xFFFFFFFFu, __vmaxu2(m, __byte_perm(m, 0u, 0x1032)));
+                }
             }
             // lane l takes row (l mod 8)'s maximum by a three-level select
             const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4;
@@ -736,8 +766,17 @@ __global__ void __launch_bounds__(kQAThreads, 2)
             uint2 cm = make_uint2(0u, 0u);  // columns (4bc, 4bc+1), (4bc+2, 4bc+3): max over the 8 rows
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                cm.x = __vmaxu2(cm.x, v[i].x & 0x7FFF7FFFu);
-                cm.y = __vmaxu2(cm.y, v[i].y & 0x7FFF7FFFu);
+                if constexpr (PROD == kProdRmsNorm) {
+                    cm.x = absmax_bf16x2(cm.x, v[i].x);
+                    cm.y = absmax_bf16x2(cm.y, v[i].y);
+                } else {
+                    cm.x = __vmaxu2(cm.x, v[i].x & 0x7FFF7FFFu);
+                    cm.y = __vmaxu2(cm.y, v[i].y & 0x7FFF7FFFu);
+                }
+            }
+            if constexpr (PROD == kProdRmsNorm) {
+                cm.x &= 0x7FFF7FFFu;
+                cm.y &= 0x7FFF7FFFu;
             }
             *reinterpret_cast<uint2 *>(&sm.col_part[br][2 * bc]) = cm;
         }
