@@ -86,8 +86,18 @@ __global__ void __launch_bounds__(kAmaxThreads, kAmaxBlocksPerSm)
     }
 }
 
+// out = 0, ahead of amax_kernel.  A kernel rather than a memset: amax_kernel,
+// launched behind it, then starts while it runs, and so does it behind the
+// kernel before.  The amax pass with a memset took 3 us more at every size (back
+// to back, us: [256, 1536] 5.2 -> 2.3, [4112, 3968] 10.4 -> 7.6).
+__global__ void amax_zero_kernel(uint32_t *__restrict__ out) {
+    pdl_wait();
+    pdl_launch_dependents();
+    *out = 0;
+}
+
 cudaError_t launch_amax(const uint16_t *x, int64_t n, uint32_t *amax, cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(amax, 0, sizeof(uint32_t), s);
+    cudaError_t e = launch_pdl(amax_zero_kernel, dim3(1), dim3(1), 0, s, amax);
     if (e != cudaSuccess || n == 0) return e;
     const int64_t nvec = n / 8;
     const int ntail = static_cast<int>(n - nvec * 8);
