@@ -11,14 +11,12 @@
 // and receives its 128 rows x BN columns of D in its own tensor memory.  Per
 // SM this halves the B bytes moved and read per MMA against a one-SM tile.
 //   warp 0      TMA producer (both CTAs): A/B tiles (128-byte swizzle) into
-//               a 3-deep ring of 256-byte K stages (two k-blocks, two swizzle
-//               atoms each), and the E8M0 scale vectors of the CTA's 128 rows
-//               of A (already in the tensor-core layout: 512 bytes per 128
-//               rows and four k-blocks); with BN = 256 also those of the
-//               tile's 256 rows of B.  Both CTAs' copies of a stage count on
-//               the even CTA's `full` barrier.  Stages of two k-blocks (eight
-//               MMAs per stage hand-off) rather than one keep the tensor pipe
-//               busy across the per-stage barrier round trip.
+//               a ring of K stages (GemmStage: six of one k-block, or four of
+//               two for 128-wide tiles), and the E8M0 scale vectors of the
+//               CTA's 128 rows of A (already in the tensor-core layout: 512
+//               bytes per 128 rows and four k-blocks); but for BN = 224 also
+//               those of the tile's rows of B.  Both CTAs' copies of a stage
+//               count on the even CTA's `full` barrier.
 //   warp 1      even CTA: MMA issuer -- copies scale vectors into tensor
 //               memory (tcgen05.cp, once per four k-blocks), issues the pair
 //               MMAs (kind::f16 / kind::f8f6f4 / kind::mxf8f6f4.block_scale,
@@ -42,10 +40,10 @@
 //                     epilogue reads the shared half first and releases the
 //                     accumulator as soon as that half is in registers, so
 //                     the next tile's MMAs wait for half a drain.
-//   block, BN = 224   two independent buffers at columns 0 and 256 (scale
+//   block, narrower   two independent buffers at columns 0 and 256 (scale
 //                     vectors at 480): the next tile never waits for a drain.
-//                     The host picks this form where the per-tile hand-off
-//                     of the 256 form would cost more than its narrower MMAs.
+//                     The host picks a narrower form where the 256-wide tiles
+//                     would leave many pairs idle (choose_tile_n).
 // Every mbarrier wait is bounded in wall time; on expiry the CTA records
 // PURO_ERR_TIMEOUT in the caller's status word, drains its own in-flight
 // copies and MMAs (with a fixed bound), and both CTAs meet at a cluster
@@ -64,10 +62,7 @@ namespace puro {
 constexpr int kBM = kGemmBM;       // rows of A per CTA (= TMEM lanes); a pair tile has 2 * kBM rows
 constexpr int kPairM = 2 * kBM;    // rows of A per pair tile
 constexpr int kAtomBytes = kGemmBKBytes;       // one 128-byte swizzle row of K: one k-block of FP8
-constexpr int kAtoms = 2;                      // k-blocks per pipeline stage
-constexpr int kBKBytes = kAtoms * kAtomBytes;  // bytes of K per pipeline stage
-constexpr int kRingBytes = 3 * 2 * kBM * kBKBytes;  // operand ring: three stages of the 256-wide form (192 KB)
-constexpr int kStagesPerGroup = 512 / kBKBytes;  // stages per group of four k-blocks (one scale chunk)
+constexpr int kRingBytes = 192 * 1024;         // operand ring
 constexpr int kThreads = 256;
 constexpr int kTmemCols = 512;
 constexpr int kSfColsPerSet = 12;  // 4 for A (128 rows) + 8 for B (up to 256 rows)
@@ -78,8 +73,6 @@ constexpr uint64_t kDrainTimeoutNs = 2000000000ull;
 constexpr uint64_t kSettleNs = 200000ull;  // after an abort: let the peer-counted copies land
 constexpr int32_t kStatusTimeout = 4;  // PURO_ERR_TIMEOUT
 constexpr int64_t kSplitRefPairs = 76;  // SM pairs the split heuristic plans for (GB300: 152 SMs)
-static_assert(kAtomBytes == 128 && kStagesPerGroup * kBKBytes == 512, "whole k-blocks per stage, whole stages per group");
-static_assert(kAtoms == 2 && kStagesPerGroup == 2, "a stage holds k-blocks 2j, 2j+1 of a group of four");
 
 // Shared memory of the quantising epilogue (kGemmOutQuant), per column
 // quarter j of the tile (64 columns, four epilogue warps q = 0..3): the row
@@ -93,12 +86,27 @@ struct QuantEpiSmem {
 };
 struct NoQuantEpiSmem {};
 
+// Pipeline stages.  A 256-wide tile's k-block keeps the tensor pipe busy for
+// 512 cycles, more than the issuing warp needs for it, so its stages are one
+// k-block and six deep: the ring then covers the copies' latency better than
+// three stages of two (61.4 against 66.6 us on [8192, 2048] x 6144, 62.6
+// against 65.6 us per-tensor on [32768, 2048] x 1536).  A 128-wide tile's takes
+// 256 cycles, about what a stage's wait, scale copies and release cost, so its
+// stages are two k-blocks (16.8 against 23.0 us on [256, 1536] x 8960).
+template <int BN>
+struct GemmStage {
+    static constexpr int kAtoms = BN == 128 ? 2 : 1;                // k-blocks (128-byte swizzle atoms) per stage
+    static constexpr int kBKBytes = kAtoms * kAtomBytes;            // bytes of K per stage
+    static constexpr int kPerGroup = 512 / kBKBytes;                // stages per group of four k-blocks (one scale chunk)
+    static constexpr int kStages = kRingBytes / ((kBM + BN / 2) * kBKBytes);  // 6, 6, 6, 4 (256, 224, 192, 128)
+    static_assert(kPerGroup * kBKBytes == 512, "whole stages per group");
+};
+
 template <int BN, bool QOUT = false>
 struct GemmSmem {
     static constexpr int kBNHalf = BN / 2;                 // rows of B per CTA
     static constexpr bool kSfbByHelper = (BN == 224);      // B scale images built by warps 2 and 3
-    // as many stages as the ring of the 256-wide form holds: 3 (256, 224, 192) or 4 (128)
-    static constexpr int kStages = kRingBytes / ((kBM + kBNHalf) * kBKBytes);
+    static constexpr int kStages = GemmStage<BN>::kStages, kAtoms = GemmStage<BN>::kAtoms;
     static constexpr int kSfbChunks = BN > 128 ? 2 : 1;    // 128-row scale chunks a tile's rows of B touch
     alignas(1024) uint8_t a[kStages][kAtoms][kBM * kAtomBytes];
     alignas(1024) uint8_t b[kStages][kAtoms][kBNHalf * kAtomBytes];
@@ -174,11 +182,13 @@ PURO_DEV void record_timeout(Smem &sm, int32_t *status) {
     if (status) atomicExch(status, kStatusTimeout);
 }
 
-// A wait of the lone issuing thread: the abort flag is read only while the
-// barrier is incomplete (an aborting role stops feeding it).
+// A wait of a whole warp, true where every lane saw the phase complete; the
+// abort flag is read only while it is incomplete (an aborting role stops
+// feeding the barrier).
 template <class Smem>
 PURO_DEV bool wait_unless_aborted(Smem &sm, uint64_t *bar, uint32_t parity, uint64_t wait_ns) {
-    return mbar_try_wait(bar, parity) || (sm.abort_flag == 0 && mbar_wait_bounded(bar, parity, wait_ns));
+    return __all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity)) ||
+           __all_sync(0xFFFFFFFFu, sm.abort_flag == 0 && mbar_wait_bounded(bar, parity, wait_ns));
 }
 
 // One unit of work: a 256 x BN pair tile and a chunk of the reduction.
@@ -521,18 +531,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                    const GemmParams p) {
     using Smem = GemmSmem<BN, OUT == kGemmOutQuant>;
     constexpr int kBNHalf = Smem::kBNHalf;
-    constexpr int kStages = Smem::kStages;
+    constexpr int kStages = Smem::kStages, kAtoms = Smem::kAtoms;
+    constexpr int kBKBytes = GemmStage<BN>::kBKBytes, kStagesPerGroup = GemmStage<BN>::kPerGroup;
     constexpr bool kMX = (KIND == kGemmFP8Block);
     constexpr bool kHelper = kMX && Smem::kSfbByHelper;
     constexpr bool OUT_F32 = (OUT == kGemmOutF32Partial || OUT == kGemmOutF32Add);
     constexpr bool OUT_Q = (OUT == kGemmOutQuant);
-    // The narrow forms run few tiles a launch: the issuing thread waits alone
-    // (a 128-wide stage's eight MMAs take 512 cycles of the tensor pipe and the
-    // waits, copies and commit of a voting warp 420 more; a 256-wide stage takes
-    // 1024 and hides them), and the epilogue arrives at the closing cluster
-    // barrier ahead of its last stores.  On the 256-wide form the former changes
-    // nothing and the latter costs 0.5%.
-    constexpr bool kLeanIssue = BN < 256 && !kHelper;
+    // The narrow forms run few tiles a launch: their epilogue arrives at the
+    // closing cluster barrier ahead of its last stores (which costs the
+    // 256-wide form 0.5%).
     constexpr bool kEarlyLeave = BN < 256 && !OUT_Q;
     constexpr bool kShifted = kMX && BN == 256;         // shared-half accumulators
     constexpr int kAccBufs = kShifted ? 1 : 2;          // hand-off barrier pairs (tfull / tempty)
@@ -553,9 +560,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
 
     extern __shared__ uint8_t smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    const int warp = threadIdx.x >> 5;
+    const int warp = __shfl_sync(0xFFFFFFFFu, static_cast<int>(threadIdx.x >> 5), 0);
     const int lane = threadIdx.x & 31;
-    const uint32_t rank = cluster_ctarank();  // 0: even CTA (issues the MMAs), 1: its peer
+    const uint32_t rank = __shfl_sync(0xFFFFFFFFu, cluster_ctarank(), 0);  // 0: even CTA (issues the MMAs), 1: its peer
     const int pair = blockIdx.x >> 1;
     const int num_pairs = gridDim.x >> 1;
 
@@ -686,7 +693,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
         }
     } else if (warp == 1 && rank == 0) {
         // ------------------------------------------------ MMA issuer (even CTA)
-        // One stage's scale copies, MMAs and release, by one thread.
+        // One stage's scale copies, MMAs and release.  The whole warp runs the
+        // loop and each instruction is predicated on the elected lane, with the
+        // warp's index and the CTA's rank broadcast above: the compiler then
+        // keeps descriptors and addresses in uniform registers.  From one lane's
+        // branch every MMA took 74 cycles to issue, for moving them there; so it
+        // takes 40 (128-wide [256, 1536] x 8960: 21.5 -> 16.8 us).
+        const uint32_t e = elect_one();
         auto issue_stage = [&](const WorkUnit &wu, int kb, uint32_t stage, uint32_t slot, uint32_t d_tmem) {
             const bool group_start = kMX && (kb % kStagesPerGroup) == 0;
             const uint32_t sfa_col = kSfBase + ((kb / kStagesPerGroup) & 1) * kSfColsPerSet;
@@ -696,10 +709,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
             if constexpr (kMX) {
                 if (group_start) {  // new group of four k-blocks: its scale vectors
                     const uint8_t *sfb_src = kHelper ? sm.sf_b[slot] : sm.sf_b[stage];
-                    tmem_cp_pair_32x128b_warpx4(tmem + sfa_col, smem_desc_plain_16B_rows(smem_u32(sm.sf_a[stage])));
-                    tmem_cp_pair_32x128b_warpx4(tmem + sfb_col, smem_desc_plain_16B_rows(smem_u32(sfb_src)));
+                    tmem_cp_pair_32x128b_warpx4_e(e, tmem + sfa_col, smem_desc_plain_16B_rows(smem_u32(sm.sf_a[stage])));
+                    tmem_cp_pair_32x128b_warpx4_e(e, tmem + sfb_col, smem_desc_plain_16B_rows(smem_u32(sfb_src)));
                     if constexpr (Smem::kSfbChunks == 2)
-                        tmem_cp_pair_32x128b_warpx4(tmem + sfb_col + 4,
+                        tmem_cp_pair_32x128b_warpx4_e(e, tmem + sfb_col + 4,
                                                     smem_desc_plain_16B_rows(smem_u32(sfb_src + 512)));
                 }
             }
@@ -718,93 +731,51 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                     const uint64_t bd = smem_desc_k_sw128(b_addr + 32 * k);
                     const uint32_t acc = (kb > wu.kb0 || at > 0 || k > 0) ? 1u : 0u;
                     if constexpr (KIND == kGemmBF16)
-                        mma_pair_f16(d_tmem, ad, bd, idesc, acc);
+                        mma_pair_f16_e(e, d_tmem, ad, bd, idesc, acc);
                     else if constexpr (KIND == kGemmFP8Tensor)
-                        mma_pair_f8(d_tmem, ad, bd, idesc, acc);
+                        mma_pair_f8_e(e, d_tmem, ad, bd, idesc, acc);
                     else
-                        mma_pair_mxf8(d_tmem, ad, bd, idesc, tmem + sfa_col, tmem + sfb_col + sfb_shift, acc);
+                        mma_pair_mxf8_e(e, d_tmem, ad, bd, idesc, tmem + sfa_col, tmem + sfb_col + sfb_shift, acc);
                 }
             }
-            tc_commit_pair_multicast(&sm.empty[stage], 0x3);  // stage reusable in both CTAs
+            tc_commit_pair_multicast_e(e, &sm.empty[stage], 0x3);  // stage reusable in both CTAs
             // the scale image is free once its copies (issued above) are done
-            if (kHelper && group_start) tc_commit_pair_multicast(&sm.sfb_empty[slot], 0x3);
+            if (kHelper && group_start) tc_commit_pair_multicast_e(e, &sm.sfb_empty[slot], 0x3);
         };
         uint32_t stage = 0, phase = 0;
-        if constexpr (kLeanIssue) {
-            if (lane == 0) {
-                bool aborted = false;
-                int local = 0;
-                PairUnits units(p, pair, num_pairs);
-                for (int u = units.next(); u >= 0 && !aborted; u = units.next(), ++local) {
-                    const WorkUnit wu = work_unit<BN>(p, u);
-                    const int buf = local % kAccBufs;
-                    const uint32_t acc_phase = static_cast<uint32_t>(local / kAccBufs) & 1u;
-                    aborted = !wait_unless_aborted(sm, &sm.tempty[buf], acc_phase ^ 1u, p.wait_ns);
-                    const uint32_t d_tmem = tmem + static_cast<uint32_t>((local & 1) * kAccShift);
-                    for (int kb = wu.kb0; kb < wu.kb1 && !aborted; ++kb) {
-                        if (!wait_unless_aborted(sm, &sm.full[stage], phase, p.wait_ns)) {
-                            aborted = true;
-                            break;
-                        }
-                        tc_fence_after_sync();
-                        issue_stage(wu, kb, stage, 0, d_tmem);
-                        if (++stage == kStages) {
-                            stage = 0;
-                            phase ^= 1u;
-                        }
-                    }
-                    if (aborted) {
-                        record_timeout(sm, p.status);
-                        break;
-                    }
-                    tc_commit_pair_multicast(&sm.tfull[buf], 0x3);  // accumulator complete in both CTAs
-                }
-            }
-            __syncwarp();
-        } else {
-            uint32_t gseq = 0;  // groups of four k-blocks started (BN = 224: slot of the scale ring)
-            bool aborted = false;
-            int local = 0;
-            PairUnits units(p, pair, num_pairs);
-            for (int u = units.next(); u >= 0 && !aborted; u = units.next(), ++local) {
-                const WorkUnit wu = work_unit<BN>(p, u);
-                const int buf = local % kAccBufs;
-                const uint32_t acc_phase = static_cast<uint32_t>(local / kAccBufs) & 1u;
-                bool ok = (sm.abort_flag == 0) && mbar_wait_bounded(&sm.tempty[buf], acc_phase ^ 1u, p.wait_ns);
-                if (!__all_sync(0xFFFFFFFFu, ok)) {
-                    if (lane == 0) record_timeout(sm, p.status);
-                    aborted = true;
-                    break;
-                }
-                tc_fence_after_sync();
-                const uint32_t d_tmem = tmem + static_cast<uint32_t>((local & 1) * kAccShift);
-                for (int kb = wu.kb0; kb < wu.kb1; ++kb) {
-                    const bool group_start = kMX && (kb % kStagesPerGroup) == 0;
-                    const uint32_t slot = gseq % kSfbSlots;
-                    ok = (sm.abort_flag == 0) && mbar_wait_bounded(&sm.full[stage], phase, p.wait_ns);
-                    if (kHelper && group_start)
-                        ok = ok && mbar_wait_bounded(&sm.sfb_full[slot], (gseq / kSfbSlots) & 1u, p.wait_ns);
-                    if (!__all_sync(0xFFFFFFFFu, ok)) {
-                        if (lane == 0) record_timeout(sm, p.status);
-                        aborted = true;
-                        break;
-                    }
-                    tc_fence_after_sync();
-                    if (lane == 0) issue_stage(wu, kb, stage, slot, d_tmem);
-                    __syncwarp();
-                    if (group_start) ++gseq;
-                    if (++stage == kStages) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
-                }
+        uint32_t gseq = 0;  // groups of four k-blocks started (BN = 224: slot of the scale ring)
+        bool aborted = false;
+        int local = 0;
+        PairUnits units(p, pair, num_pairs);
+        for (int u = units.next(); u >= 0 && !aborted; u = units.next(), ++local) {
+            const WorkUnit wu = work_unit<BN>(p, u);
+            const int buf = local % kAccBufs;
+            const uint32_t acc_phase = static_cast<uint32_t>(local / kAccBufs) & 1u;
+            aborted = !wait_unless_aborted(sm, &sm.tempty[buf], acc_phase ^ 1u, p.wait_ns);
+            const uint32_t d_tmem = tmem + static_cast<uint32_t>((local & 1) * kAccShift);
+            for (int kb = wu.kb0; kb < wu.kb1 && !aborted; ++kb) {
+                const bool group_start = kMX && (kb % kStagesPerGroup) == 0;
+                const uint32_t slot = gseq % kSfbSlots;
+                aborted = !wait_unless_aborted(sm, &sm.full[stage], phase, p.wait_ns) ||
+                          (kHelper && group_start &&
+                           !wait_unless_aborted(sm, &sm.sfb_full[slot], (gseq / kSfbSlots) & 1u, p.wait_ns));
                 if (aborted) break;
-                if (lane == 0) tc_commit_pair_multicast(&sm.tfull[buf], 0x3);  // accumulator complete in both CTAs
-                __syncwarp();
+                tc_fence_after_sync();
+                issue_stage(wu, kb, stage, slot, d_tmem);
+                if (group_start) ++gseq;
+                if (++stage == kStages) {
+                    stage = 0;
+                    phase ^= 1u;
+                }
             }
+            if (aborted) {
+                if (lane == 0) record_timeout(sm, p.status);
+                break;
+            }
+            tc_commit_pair_multicast_e(e, &sm.tfull[buf], 0x3);  // accumulator complete in both CTAs
         }
         // All MMAs and copies issued by this warp complete before teardown.
-        if (lane == 0) {
+        if (e) {
             tc_commit_pair(&sm.drain);
             mbar_wait_bounded(&sm.drain, 0, kDrainTimeoutNs);
         }
@@ -1095,23 +1066,22 @@ int choose_splits(int64_t M, int64_t N, int64_t K, bool bf16) {
 }
 
 // Modelled cycles of one tile: a pair MMA (32 bytes of K) and the tile's
-// hand-off.  Fitted to GB300 times of the three widths over fifteen shapes from
-// [256, 1536] to [32768, 2048], K = 1536 .. 8960, back to back.  The narrower
-// MMAs are bound by the operands' way into shared memory, not by the tensor
-// pipe (a 128-wide one would take 64 cycles there), so a narrow tile is no
-// faster per column; it pays where it fits the same number of rounds, that is
-// where the 256-wide tiles leave many SM pairs idle.  Block-scaled, us at 256 /
-// 192 / 128: [256, 1536, K 1536] 8.0 / 7.5 / 6.8, [256, 1536, 8960] 25.7 /
-// 23.7 / 22.2, [1024, 2048, 2048] 9.9 / 9.8 / 8.8, [2048, 1536, 1536] 9.3 /
-// 8.7 / 11.1; but [2048, 2048, 2048] 10.8 / 14.8 / 13.5 and [8192, 2048, 2048]
-// 27 / 30 / 37.
+// hand-off.  Fitted to GB300 times of the three widths over sixteen shapes from
+// [256, 1536] to [32768, 2048], K = 1536 .. 8960, back to back.  A 192-wide MMA
+// takes nearly as long as a 256-wide one and a 128-wide one more than half, so
+// the narrow tiles are no faster per column; they pay where they need no more
+// rounds, that is where the 256-wide tiles leave many SM pairs idle.
+// Block-scaled, us at 256 / 192 / 128: [256, 1536, K 1536] 7.8 / 7.4 / 5.6,
+// [256, 1536, 8960] 23.6 / 22.1 / 16.8, [1024, 2048, 2048] 9.4 / 9.1 / 7.0,
+// [2048, 1536, 1536] 8.7 / 8.2 / 8.9, [4096, 1536, 8960] 44.0 / 41.8 / 44.6; but
+// [4096, 2048, 2048] 15.6 / 19.0 / 17.9 and [8192, 2048, 2048] 25.8 / 28.9 / 28.9.
 struct TileCost {
     int width, per_mma, per_tile;
 };
-constexpr TileCost kTileCosts[] = {{256, 147, 600}, {192, 135, 400}, {128, 125, 350}};
+constexpr TileCost kTileCosts[] = {{256, 131, 900}, {192, 120, 500}, {128, 95, 400}};
 
 static int64_t tile_cycles(const TileCost &c, int64_t red) {
-    return (red + kBKBytes - 1) / kBKBytes * kAtoms * 4 * c.per_mma + c.per_tile;
+    return (red + kAtomBytes - 1) / kAtomBytes * (kAtomBytes / 32) * c.per_mma + c.per_tile;
 }
 static int64_t pair_tiles(int64_t rows, int64_t cols, int64_t width) {
     return (rows + kPairM - 1) / kPairM * ((cols + width - 1) / width);
@@ -1137,8 +1107,8 @@ int choose_tile_n(int64_t M, int64_t N, int64_t K) {
 // Tile width of a linear's Dgrad (dX [M, K], reduction N) and Wgrad (dW [N, K],
 // reduction M) in one grouped launch: the modelled makespan of the balanced
 // schedule, the longer reduction's tiles first.  Measured at 256 / 192 / 128,
-// us: (M, N, K) = (256, 1536, 1536) 8.1 / 7.6 / 6.8, (640, 1152, 2560) 9.0 /
-// 9.8 / 10.0, (2048, 2048, 2048) 15.9 / 19.4 / 22.1.
+// us: (M, N, K) = (256, 1536, 1536) 7.8 / 7.4 / 5.6, (640, 1152, 2560) 8.4 /
+// 8.8 / 8.8, (2048, 2048, 2048) 15.1 / 18.7 / 17.3.
 int choose_grouped_tile_n(int64_t M, int64_t N, int64_t K) {
     int best = 256;
     int64_t best_cost = 0;
@@ -1197,7 +1167,8 @@ static int max_resident_pairs(int num_sms, size_t smem) {
 template <int KIND, int OUT, int BN>
 static GemmParams make_params(const GemmArgs &g, int splits) {
     constexpr int kElemBytes = (KIND == kGemmBF16) ? 2 : 1;
-    constexpr int kBK = kBKBytes / kElemBytes;
+    constexpr int kBK = GemmStage<BN>::kBKBytes / kElemBytes;
+    constexpr int kStagesPerGroup = GemmStage<BN>::kPerGroup;
     GemmParams p{};
     p.M = static_cast<int>(g.M);
     p.N = static_cast<int>(g.N);
@@ -1322,22 +1293,22 @@ cudaError_t launch_gemm_grouped(const GemmArgs &g0, const GemmMaps &m0, const Ge
     }
 }
 
-// Modelled time, in pipeline stages of one pair, of a linear's Dgrad and
+// Modelled time, in units of two k-blocks of one pair, of a linear's Dgrad and
 // Wgrad as one grouped launch with the balanced schedule (the longer
 // reduction's tiles first), against separate launches where the Wgrad
 // splits its reduction into `w_splits` chunks (plus its reduction kernel and
-// launch, about 20 stages).  Host-only, shape-only.
+// launch, about 20 units).  Host-only, shape-only.
 bool grouped_backward_faster(int64_t M, int64_t N, int64_t K, int w_splits) {
     const int64_t P = kSplitRefPairs;
     auto tiles = [](int64_t r, int64_t c) { return ((r + kPairM - 1) / kPairM) * ((c + 255) / 256); };
-    auto stages = [](int64_t red) { return (red + kBKBytes - 1) / kBKBytes; };
+    auto stages = [](int64_t red) { return (red + 255) / 256; };
     const int64_t ud = tiles(M, K), ld = stages(N);  // Dgrad: dX [M, K], reduction N
     const int64_t uw = tiles(N, K), lw = stages(M);  // Wgrad: dW [N, K], reduction M
     const int64_t u0 = ld >= lw ? ud : uw, l0 = ld >= lw ? ld : lw;
     const int64_t u1 = ld >= lw ? uw : ud, l1 = ld >= lw ? lw : ld;
     const int64_t grouped = std::max((u0 + P - 1) / P * l0, (u0 * l0 + u1 * l1 + P - 1) / P + l1);
     if (w_splits <= 1) return true;  // both unsplit: one launch, no worse than two
-    const int64_t chunk = ((lw + w_splits - 1) / w_splits + kStagesPerGroup - 1) / kStagesPerGroup * kStagesPerGroup;
+    const int64_t chunk = ((lw + w_splits - 1) / w_splits + 1) / 2 * 2;
     const int64_t separate = (ud + P - 1) / P * ld + (uw * w_splits + P - 1) / P * chunk + 20;
     return grouped < separate;
 }
