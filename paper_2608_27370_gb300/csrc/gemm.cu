@@ -626,69 +626,69 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
-        if (lane == 0) {
-            const uint32_t full0 = mapa_shared(smem_u32(&sm.full[0]), 0);  // the even CTA's ring
-            uint32_t stage = 0, phase = 0;
-            uint32_t issued = 0;  // stage fills started by this thread
-            bool aborted = false;
-            PairUnits units(p, pair, num_pairs);
-            for (int u = units.next(); u >= 0 && !aborted; u = units.next()) {
-                const WorkUnit wu = work_unit<BN>(p, u);
-                const int a_row = wu.m0 + kBM * static_cast<int>(rank);
-                const int b_row = wu.n0 + kBNHalf * static_cast<int>(rank);
-                const CUtensorMap *ma = wu.problem ? &tm_a1 : &tm_a;
-                const CUtensorMap *mb = wu.problem ? &tm_b1 : &tm_b;
-                const CUtensorMap *msfa = wu.problem ? &tm_sfa1 : &tm_sfa;
-                const CUtensorMap *msfb = wu.problem ? &tm_sfb1 : &tm_sfb;
-                const int kgroups = wu.problem ? p.kgroups1 : p.kgroups;
-                for (int kb = wu.kb0; kb < wu.kb1; ++kb) {
-                    if (sm.abort_flag || !mbar_wait_bounded(&sm.empty[stage], phase ^ 1u, p.wait_ns)) {
-                        record_timeout(sm, p.status);
-                        aborted = true;
-                        break;
-                    }
-                    const bool sf_load = kMX && (kb % kStagesPerGroup) == 0;
-                    const uint32_t full_bar = full0 + 8u * stage;
-                    if (rank == 0)
-                        mbar_arrive_expect_tx(&sm.full[stage], 2u * (kStageBytes + (sf_load ? kSfBytes : 0u)));
+        // (the whole warp, as the MMA issuer: see there)
+        const uint32_t e = elect_one();
+        const uint32_t full0 = mapa_shared(smem_u32(&sm.full[0]), 0);  // the even CTA's ring
+        uint32_t stage = 0, phase = 0;
+        uint32_t issued = 0;  // stage fills started
+        bool aborted = false;
+        PairUnits units(p, pair, num_pairs);
+        for (int u = units.next(); u >= 0 && !aborted; u = units.next()) {
+            const WorkUnit wu = work_unit<BN>(p, u);
+            const int a_row = wu.m0 + kBM * static_cast<int>(rank);
+            const int b_row = wu.n0 + kBNHalf * static_cast<int>(rank);
+            const CUtensorMap *ma = wu.problem ? &tm_a1 : &tm_a;
+            const CUtensorMap *mb = wu.problem ? &tm_b1 : &tm_b;
+            const CUtensorMap *msfa = wu.problem ? &tm_sfa1 : &tm_sfa;
+            const CUtensorMap *msfb = wu.problem ? &tm_sfb1 : &tm_sfb;
+            const int kgroups = wu.problem ? p.kgroups1 : p.kgroups;
+            for (int kb = wu.kb0; kb < wu.kb1; ++kb) {
+                if (!wait_unless_aborted(sm, &sm.empty[stage], phase ^ 1u, p.wait_ns)) {
+                    if (lane == 0) record_timeout(sm, p.status);
+                    aborted = true;
+                    break;
+                }
+                const bool sf_load = kMX && (kb % kStagesPerGroup) == 0;
+                const uint32_t full_bar = full0 + 8u * stage;
+                if (rank == 0 && e)
+                    mbar_arrive_expect_tx(&sm.full[stage], 2u * (kStageBytes + (sf_load ? kSfBytes : 0u)));
 #pragma unroll
-                    for (int at = 0; at < kAtoms; ++at) {
-                        tma_load_2d_pair(sm.a[stage][at], ma, full_bar, kb * kBK + at * kAtomK, a_row);
-                        tma_load_2d_pair(sm.b[stage][at], mb, full_bar, kb * kBK + at * kAtomK, b_row);
+                for (int at = 0; at < kAtoms; ++at) {
+                    tma_load_2d_pair_e(e, sm.a[stage][at], ma, full_bar, kb * kBK + at * kAtomK, a_row);
+                    tma_load_2d_pair_e(e, sm.b[stage][at], mb, full_bar, kb * kBK + at * kAtomK, b_row);
+                }
+                if (sf_load) {
+                    // chunks beyond the operand's rows read as zero (their rows are zero too)
+                    const int kg = kb / kStagesPerGroup;
+                    tma_load_2d_pair_e(e, sm.sf_a[stage], msfa, full_bar, 0, (a_row / 128) * kgroups + kg);
+                    if constexpr (!kHelper) {
+                        tma_load_2d_pair_e(e, sm.sf_b[stage], msfb, full_bar, 0, (wu.n0 / 128) * kgroups + kg);
+                        if constexpr (Smem::kSfbChunks == 2)
+                            tma_load_2d_pair_e(e, sm.sf_b[stage] + 512, msfb, full_bar, 0,
+                                             (wu.n0 / 128 + 1) * kgroups + kg);
                     }
-                    if (sf_load) {
-                        // chunks beyond the operand's rows read as zero (their rows are zero too)
-                        const int kg = kb / kStagesPerGroup;
-                        tma_load_2d_pair(sm.sf_a[stage], msfa, full_bar, 0, (a_row / 128) * kgroups + kg);
-                        if constexpr (!kHelper) {
-                            tma_load_2d_pair(sm.sf_b[stage], msfb, full_bar, 0, (wu.n0 / 128) * kgroups + kg);
-                            if constexpr (Smem::kSfbChunks == 2)
-                                tma_load_2d_pair(sm.sf_b[stage] + 512, msfb, full_bar, 0,
-                                                 (wu.n0 / 128 + 1) * kgroups + kg);
-                        }
-                    }
-                    ++issued;
-                    if (++stage == kStages) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
+                }
+                ++issued;
+                if (++stage == kStages) {
+                    stage = 0;
+                    phase ^= 1u;
                 }
             }
-            if (rank == 0) {
-                // Every fill of the ring (both CTAs' copies) lands before the
-                // pair exits: wait for the latest fill of each stage.
-                for (uint32_t s = 0; s < kStages; ++s) {
-                    const uint32_t fills = issued / kStages + (s < issued % kStages ? 1u : 0u);
-                    if (fills > 0) mbar_wait_bounded(&sm.full[s], (fills - 1u) & 1u, kDrainTimeoutNs);
-                }
+        }
+        if (rank == 0) {
+            // Every fill of the ring (both CTAs' copies) lands before the
+            // pair exits: wait for the latest fill of each stage.
+            for (uint32_t s = 0; s < kStages; ++s) {
+                const uint32_t fills = issued / kStages + (s < issued % kStages ? 1u : 0u);
+                if (fills > 0) mbar_wait_bounded(&sm.full[s], (fills - 1u) & 1u, kDrainTimeoutNs);
             }
-            if (aborted) {
-                // This CTA's copies count on the even CTA's barriers, so it
-                // cannot wait for them itself: give any still in flight a
-                // fixed time to land.
-                const uint64_t t0 = global_timer_ns();
-                while (global_timer_ns() - t0 < kSettleNs) {
-                }
+        }
+        if (aborted) {
+            // This CTA's copies count on the even CTA's barriers, so it
+            // cannot wait for them itself: give any still in flight a
+            // fixed time to land.
+            const uint64_t t0 = global_timer_ns();
+            while (global_timer_ns() - t0 < kSettleNs) {
             }
         }
     } else if (warp == 1 && rank == 0) {
@@ -698,7 +698,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
         // warp's index and the CTA's rank broadcast above: the compiler then
         // keeps descriptors and addresses in uniform registers.  From one lane's
         // branch every MMA took 74 cycles to issue, for moving them there; so it
-        // takes 40 (128-wide [256, 1536] x 8960: 21.5 -> 16.8 us).
+        // takes 40 (128-wide [256, 1536] x 8960: 21.5 -> 16.8 us).  The producer's
+        // copies and the epilogue's stores are issued the same way (together
+        // 2-10%: [32768, 2048] x 1536 71.9 -> 68.4 us, grouped backward of
+        // (640, 1152, 2560) 11.1 -> 10.0).
         const uint32_t e = elect_one();
         auto issue_stage = [&](const WorkUnit &wu, int kb, uint32_t stage, uint32_t slot, uint32_t d_tmem) {
             const bool group_start = kMX && (kb % kStagesPerGroup) == 0;
@@ -839,6 +842,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
     } else if (warp >= 4) {
         // ------------------------------------------------ epilogue (both CTAs)
         const int q = warp & 3;  // TMEM lane quarter of this warp
+        const uint32_t e = elect_one();
         float sab = 1.0f;
         if constexpr (KIND == kGemmFP8Tensor) sab = __fmul_rn(*p.sia, *p.sib);
         uint8_t *stage_buf = sm.epi[q];
@@ -900,7 +904,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                     for (int c = 0; c < 4; ++c) {
                         const int col = n0 + 128 * h + 32 * c;
                         if (c >= nc || col >= n_out) break;
-                        if (lane == 0) bulk_wait_group_read0();
+                        if (e) bulk_wait_group_read0();
                         __syncwarp();
                         uint8_t *row = stage_buf + 128 * lane;
 #pragma unroll
@@ -916,7 +920,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                         }
                         fence_proxy_async_smem();
                         __syncwarp();
-                        if (lane == 0) {
+                        if (e) {
                             if constexpr (OUT == kGemmOutF32Add)
                                 tma_reduce_add_2d(md, stage_buf, col, row0);
                             else
@@ -951,7 +955,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                         const int col = n0 + 128 * h + 32 * c;
                         if (c >= nc || col >= n_out) break;
                         uint8_t *half = stage_buf + 2048 * (pieces & 1u);
-                        if (lane == 0) bulk_wait_group_read<1>();  // the store that last read this half is done
+                        if (e) bulk_wait_group_read<1>();  // the store that last read this half is done
                         __syncwarp();
                         uint8_t *row = half + 64 * lane;
 #pragma unroll
@@ -962,16 +966,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                         }
                         fence_proxy_async_smem();
                         __syncwarp();
-                        if (lane == 0) {
-                            tma_store_2d(md, half, col, m0 + 32 * q);
-                            bulk_commit_group();
-                        }
+                        tma_store_2d_e(e, md, half, col, m0 + 32 * q);
                         ++pieces;
                     }
                 }
             }
         }
-        if (lane == 0) bulk_wait_group0();
+        if (e) bulk_wait_group0();
         __syncwarp();
     }
 

@@ -21,6 +21,15 @@ PURO_DEV uint32_t lane_id() {
     return l;
 }
 
+// 1 in one lane of the warp (always the same one), 0 in the others.  The forms
+// below with a suffix _e are run by a whole warp and take effect in that lane,
+// so that their operands can stay in uniform registers.
+PURO_DEV uint32_t elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r;
+}
+
 PURO_DEV uint64_t global_timer_ns() {
     uint64_t t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -140,6 +149,16 @@ PURO_DEV void tma_store_2d(const CUtensorMap *map, const void *src, int32_t x, i
                  : "memory");
 }
 
+// (with its commit)
+PURO_DEV void tma_store_2d_e(uint32_t e, const CUtensorMap *map, const void *src, int32_t x, int32_t y) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %4, 0;\n\t"
+        "@q cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];\n\t"
+        "@q cp.async.bulk.commit_group;\n\t}" ::"l"(reinterpret_cast<uint64_t>(map)),
+        "r"(smem_u32(src)), "r"(x), "r"(y), "r"(e)
+        : "memory");
+}
+
 // 2-D tiled element-wise add shared -> global (bulk-group completion): each
 // element of the box is added to the global tensor's element (the tensor
 // map's type; f32 adds round to nearest).
@@ -234,11 +253,14 @@ PURO_DEV void mbar_arrive_cluster_cta_scope(uint32_t bar_cluster) {
 
 // 2-D tiled load into this CTA's shared memory whose completion is counted
 // on an mbarrier that may live in the peer CTA of the pair.
-PURO_DEV void tma_load_2d_pair(void *dst, const CUtensorMap *map, uint32_t bar_cluster, int32_t x, int32_t y) {
+
+PURO_DEV void tma_load_2d_pair_e(uint32_t e, void *dst, const CUtensorMap *map, uint32_t bar_cluster, int32_t x,
+                                 int32_t y) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
-        " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar_cluster)
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+        "@q cp.async.bulk.tensor.2d.shared::cta.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
+        " [%0], [%1, {%2, %3}], [%4];\n\t}" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar_cluster), "r"(e)
         : "memory");
 }
 
@@ -296,28 +318,24 @@ PURO_DEV void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&r)[32]) {
 }
 PURO_DEV void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// ---- the same issued by a whole warp for its elected lane (e: this lane is it)
-PURO_DEV uint32_t elect_one() {
-    uint32_t r;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
-    return r;
-}
-PURO_DEV void mma_pair_f16_e(uint32_t e, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+PURO_DEV void mma_pair_f16_e(uint32_t e, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                             uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
         "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(e)
         : "memory");
 }
-PURO_DEV void mma_pair_f8_e(uint32_t e, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+PURO_DEV void mma_pair_f8_e(uint32_t e, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                            uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
         "@q tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(e)
         : "memory");
 }
-PURO_DEV void mma_pair_mxf8_e(uint32_t e, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t sfa_tmem,
-                            uint32_t sfb_tmem, uint32_t accumulate) {
+PURO_DEV void mma_pair_mxf8_e(uint32_t e, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                              uint32_t sfa_tmem, uint32_t sfb_tmem, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %7, 0;\n\t"
         "@q tcgen05.mma.cta_group::2.kind::mxf8f6f4.block_scale.scale_vec::1X [%0], %1, %2, %3, [%5], [%6], p;\n\t}\n" ::"r"(
@@ -326,11 +344,16 @@ PURO_DEV void mma_pair_mxf8_e(uint32_t e, uint32_t d_tmem, uint64_t adesc, uint6
         : "memory");
 }
 PURO_DEV void tmem_cp_pair_32x128b_warpx4_e(uint32_t e, uint32_t taddr, uint64_t sdesc) {
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q tcgen05.cp.cta_group::2.32x128b.warpx4 [%0], %1;\n\t}" ::"r"(taddr), "l"(sdesc), "r"(e) : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q tcgen05.cp.cta_group::2.32x128b.warpx4 [%0], %1;\n\t}" ::"r"(
+            taddr),
+        "l"(sdesc), "r"(e)
+        : "memory");
 }
 PURO_DEV void tc_commit_pair_multicast_e(uint32_t e, uint64_t *bar, uint16_t cta_mask) {
     asm volatile(
-        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(
+        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+        "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(
             smem_u32(bar)),
         "h"(cta_mask), "r"(e)
         : "memory");
