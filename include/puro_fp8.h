@@ -263,9 +263,10 @@ puro_status_t puro_swiglu_bf16(const void *gate, const void *up, int64_t rows, i
  *   workspace, workspace_bytes: optional scratch (may be NULL/0), 16-byte
  *     aligned.  When the output has fewer 128x256 tiles than the GPU has
  *     SMs and at least puro_fp8_workspace_size(...) bytes are given, the
- *     reduction is split into chunks whose FP32 partial tiles go to the
- *     workspace and are summed (in fixed chunk order, then rounded once to
- *     BF16) by a second kernel on the same stream.  Results are within the
+ *     reduction is split into chunks whose FP32 partial tiles are summed in
+ *     fixed chunk order, then rounded once to BF16: inside clusters of the
+ *     one launch where the output has few tiles, else through the workspace
+ *     by a second kernel on the same stream.  Results are within the
  *     output tolerance either way, and deterministic for a given split.
  *     The workspace is only written, never read before being written.
  *   dev_status: optional device int32, written only on a device-side
@@ -396,7 +397,7 @@ puro_status_t puro_fp8_linear_wgrad_noalloc(const puro_fp8_tensor_t *dy_t, const
  * Kernel launches puro_fp8_linear_backward makes for block-scaled operands
  * of a linear with M tokens, N output and K input features, given
  * workspace_bytes of (16-byte aligned) workspace: 1 for a grouped launch,
- * else one per GEMM plus one per split reduction.  0 for an empty extent.
+ * else one per GEMM plus one per reduction split through the workspace.  0 for an empty extent.
  * Host-only, no CUDA call.
  */
 int32_t puro_fp8_linear_backward_launches(int64_t M, int64_t N, int64_t K, size_t workspace_bytes);

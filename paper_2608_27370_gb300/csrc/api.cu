@@ -137,7 +137,8 @@ puro_status_t prepare_fp8_gemm(const puro_fp8_tensor_t *a, const puro_fp8_tensor
     const int sp = choose_splits(M, N, K, false);
     const bool split = sp > 1 && workspace && aligned16(workspace) &&
                        workspace_bytes >= splitk_workspace_bytes(M, N, K, false);
-    const int tile_n = split ? 256 : width ? width : tile_width(block ? kGemmFP8Block : kGemmFP8Tensor, accumulate_f32, M, N, K);
+    const int cluster = split ? cluster_split(M, N, K, sp) : 1;
+    const int tile_n = cluster > 1 ? 128 : split ? 256 : width ? width : tile_width(block ? kGemmFP8Block : kGemmFP8Tensor, accumulate_f32, M, N, K);
 
     GemmMaps m{};
     if (!make_map(&m.a, CU_TENSOR_MAP_DATA_TYPE_UINT8, a->data, K, M, K, kGemmBKBytes, kGemmBM,
@@ -171,14 +172,14 @@ puro_status_t prepare_fp8_gemm(const puro_fp8_tensor_t *a, const puro_fp8_tensor
     g.num_sms = sm_count();
     if (g.num_sms <= 0) return PURO_ERR_CUDA;
     g.out = d;
-    g.splits = 1;
+    g.splits = split ? sp : 1;
+    g.cluster = cluster;
     g.accumulate_f32 = accumulate_f32;
-    if (split) {
+    if (split && cluster == 1) {
         const uint64_t rows = static_cast<uint64_t>(sp) * static_cast<uint64_t>(splitk_rows_per_chunk(M));
         if (!make_map(&m.ws, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, workspace, N, rows, N * 4, 32, 32,
                       CU_TENSOR_MAP_SWIZZLE_128B))
             return PURO_ERR_CUDA;
-        g.splits = sp;
         g.workspace = workspace;
     }
     *gout = g;
@@ -230,7 +231,10 @@ BackwardPlan plan_backward(int64_t M, int64_t N, int64_t K, size_t ws) {
         else
             b.grouped = b.wgrad_unsplit = grouped_backward_faster(M, N, K, sw);
     }
-    b.launches = b.grouped ? 1 : (sd > 1 ? 2 : 1) + (sw > 1 ? 2 : 1);
+    auto launches_of = [](int sp, int64_t r, int64_t c, int64_t red) {
+        return sp > 1 && cluster_split(r, c, red, sp) == 1 ? 2 : 1;
+    };
+    b.launches = b.grouped ? 1 : launches_of(sd, M, K, N) + launches_of(sw, N, K, M);
     return b;
 }
 

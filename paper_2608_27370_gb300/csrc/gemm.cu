@@ -104,11 +104,21 @@ struct GemmStage {
     static_assert(kPerGroup * kBKBytes == 512, "whole stages per group");
 };
 
-template <int BN, bool QOUT = false>
+// Partial slices of the tile from the other pairs of its cluster (S pairs share
+// the reduction): per pair 128 rows x 128 / S columns of FP32, 16-byte chunk i
+// of row r at i ^ (r % 8).
+template <int S>
+struct SplitSmem {
+    alignas(1024) uint8_t part[S - 1][kBM * 128 / S * 4];
+};
+struct NoSplitSmem {};
+
+template <int BN, bool QOUT = false, int S = 1>
 struct GemmSmem {
     static constexpr int kBNHalf = BN / 2;                 // rows of B per CTA
     static constexpr bool kSfbByHelper = (BN == 224);      // B scale images built by warps 2 and 3
-    static constexpr int kStages = GemmStage<BN>::kStages, kAtoms = GemmStage<BN>::kAtoms;
+    // (a stage of the ring makes room for the partial slices)
+    static constexpr int kStages = GemmStage<BN>::kStages - (S > 1 ? 1 : 0), kAtoms = GemmStage<BN>::kAtoms;
     static constexpr int kSfbChunks = BN > 128 ? 2 : 1;    // 128-row scale chunks a tile's rows of B touch
     alignas(1024) uint8_t a[kStages][kAtoms][kBM * kAtomBytes];
     alignas(1024) uint8_t b[kStages][kAtoms][kBNHalf * kAtomBytes];
@@ -130,6 +140,7 @@ struct GemmSmem {
     uint32_t tmem_base;
     volatile int abort_flag;
     std::conditional_t<QOUT, QuantEpiSmem, NoQuantEpiSmem> qe;
+    std::conditional_t<(S > 1), SplitSmem<S>, NoSplitSmem> split;
 };
 
 struct GemmParams {
@@ -526,15 +537,20 @@ PURO_DEV void quant_epilogue(Smem &sm, const GemmParams &p, uint32_t tmem, int w
 template <int OUT>
 constexpr int gemm_threads() { return OUT == kGemmOutQuant ? kThreads + 384 : kThreads; }
 
-template <int KIND, int OUT, int BN>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(), 1)
+// S > 1: S pairs of a cluster share one 128-wide tile, each a part of its
+// reduction.  Each CTA then hands the columns that another pair finishes to
+// that pair's CTA of the same rows, through distributed shared memory, and adds
+// up its own 128 / S columns in pair order.  One launch and no scratch, for
+// outputs of few tiles: see cluster_split.
+template <int KIND, int OUT, int BN, int S = 1>
+__global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT>(), 1)
     gemm_tn_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                    const __grid_constant__ CUtensorMap tm_d, const __grid_constant__ CUtensorMap tm_sfa,
                    const __grid_constant__ CUtensorMap tm_sfb, const __grid_constant__ CUtensorMap tm_a1,
                    const __grid_constant__ CUtensorMap tm_b1, const __grid_constant__ CUtensorMap tm_d1,
                    const __grid_constant__ CUtensorMap tm_sfa1, const __grid_constant__ CUtensorMap tm_sfb1,
                    const GemmParams p) {
-    using Smem = GemmSmem<BN, OUT == kGemmOutQuant>;
+    using Smem = GemmSmem<BN, OUT == kGemmOutQuant, S>;
     constexpr int kBNHalf = Smem::kBNHalf;
     constexpr int kStages = Smem::kStages, kAtoms = Smem::kAtoms;
     constexpr int kBKBytes = GemmStage<BN>::kBKBytes, kStagesPerGroup = GemmStage<BN>::kPerGroup;
@@ -562,7 +578,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
     constexpr uint32_t kSfBytes = kHelper ? 512u : 512u + 512u * Smem::kSfbChunks;  // one CTA's TMA scale bytes per group
     static_assert(BN == 256 || BN == 192 || BN == 128 || (BN == 224 && kMX && OUT == kGemmOutBF16),
                   "the 224-wide form is block-scaled, BF16 out");
-    static_assert(OUT != kGemmOutF32Partial || BN == 256, "split reductions run 256-wide");
+    static_assert(OUT != kGemmOutF32Partial || BN == 256, "reductions split through memory run 256-wide");
+    static_assert(S == 1 || (BN == 128 && KIND != kGemmBF16 && OUT != kGemmOutF32Partial), "128-wide FP8 tiles");
     static_assert(!OUT_Q || (kMX && BN == 256), "the quantising epilogue is block-scaled and 256-wide");
     static_assert(!kMX || kSfBase + kSfSets * kSfColsPerSet <= kTmemCols, "TMEM budget");
     static_assert(kAccShift + BN <= (kMX ? kSfBase : kTmemCols), "accumulators clear of the scale columns");
@@ -571,9 +588,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
     Smem &sm = *reinterpret_cast<Smem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int warp = __shfl_sync(0xFFFFFFFFu, static_cast<int>(threadIdx.x >> 5), 0);
     const int lane = threadIdx.x & 31;
-    const uint32_t rank = __shfl_sync(0xFFFFFFFFu, cluster_ctarank(), 0);  // 0: even CTA (issues the MMAs), 1: its peer
-    const int pair = blockIdx.x >> 1;
-    const int num_pairs = gridDim.x >> 1;
+    const uint32_t crank = __shfl_sync(0xFFFFFFFFu, cluster_ctarank(), 0);
+    const uint32_t rank = S == 1 ? crank : crank & 1u;  // 0: even CTA (issues the MMAs), 1: its peer
+    const uint32_t even = crank - rank;                 // the pair's even CTA in the cluster
+    const int part = static_cast<int>(crank >> 1);      // the pair's part of the reduction (S > 1)
+    const uint16_t both = static_cast<uint16_t>(0x3u << even);
+    const int pair = blockIdx.x / (2 * S);              // (S > 1: the cluster)
+    const int num_pairs = gridDim.x / (2 * S);
+    auto unit = [&](int u) {
+        WorkUnit w = work_unit<BN>(p, u);
+        if constexpr (S > 1) {
+            w.kb0 = p.num_kb * part / S;
+            w.kb1 = p.num_kb * (part + 1) / S;
+        }
+        return w;
+    };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -622,7 +651,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
     const uint32_t tmem = warp != 0 ? sm.tmem_base : 0u;
     // Arrive at the closing cluster barrier: this warp is done with tensor
     // memory and the peer's barriers.
-    bool left = false;
+    bool left = false, met = false;  // (met: it has waited there)
     auto leave = [&] {
         tc_fence_before_sync();
         __syncwarp();
@@ -635,13 +664,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
         // ------------------------------------------------ TMA producer
         // (the whole warp, as the MMA issuer: see there)
         const uint32_t e = elect_one();
-        const uint32_t full0 = mapa_shared(smem_u32(&sm.full[0]), 0);  // the even CTA's ring
+        const uint32_t full0 = mapa_shared(smem_u32(&sm.full[0]), even);  // the even CTA's ring
         uint32_t stage = 0, phase = 0;
         uint32_t issued = 0;  // stage fills started
         bool aborted = false;
         PairUnits units(p, pair, num_pairs);
         for (int u = units.next(); u >= 0 && !aborted; u = units.next()) {
-            const WorkUnit wu = work_unit<BN>(p, u);
+            const WorkUnit wu = unit(u);
             const int a_row = wu.m0 + kBM * static_cast<int>(rank);
             const int b_row = wu.n0 + kBNHalf * static_cast<int>(rank);
             const CUtensorMap *ma = wu.problem ? &tm_a1 : &tm_a;
@@ -655,7 +684,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                     aborted = true;
                     break;
                 }
-                const bool sf_load = kMX && (kb % kStagesPerGroup) == 0;
+                const bool sf_load = kMX && ((kb % kStagesPerGroup) == 0 || (S > 1 && kb == wu.kb0));
                 const uint32_t full_bar = full0 + 8u * stage;
                 if (rank == 0 && e)
                     mbar_arrive_expect_tx(&sm.full[stage], 2u * (kStageBytes + (sf_load ? kSfBytes : 0u)));
@@ -765,7 +794,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
         int local = 0;
         PairUnits units(p, pair, num_pairs);
         for (int u = units.next(); u >= 0 && !aborted; u = units.next(), ++local) {
-            const WorkUnit wu = work_unit<BN>(p, u);
+            const WorkUnit wu = unit(u);
             const int buf = local % kAccBufs;
             const uint32_t acc_phase = static_cast<uint32_t>(local / kAccBufs) & 1u;
             aborted = !wait_unless_aborted(sm, &sm.tempty[buf], acc_phase ^ 1u, p.wait_ns);
@@ -776,7 +805,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
             const int kt = kTail > 0 ? max(wu.kb0, wu.kb1 - kTail) : wu.kb1;
             // the operands of stage kb, and its group's scales, are there
             auto stage_ready = [&](int kb) {
-                const bool group_start = kMX && (kb % kStagesPerGroup) == 0;
+                const bool group_start = kMX && ((kb % kStagesPerGroup) == 0 || (S > 1 && kb == wu.kb0));
                 const uint32_t slot = gseq % kSfbSlots;
                 if (!wait_unless_aborted(sm, &sm.full[stage], phase, p.wait_ns)) return false;
                 if (kHelper && group_start &&
@@ -798,10 +827,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                     break;
                 }
                 issue_mmas(wu, kb, stage, d_tmem, idesc, 0, sfb_shift);
-                tc_commit_pair_multicast_e(e, &sm.empty[stage], 0x3);  // stage reusable in both CTAs
+                tc_commit_pair_multicast_e(e, &sm.empty[stage], both);  // stage reusable in both CTAs
                 if (kHelper && (kb % kStagesPerGroup) == 0) {
                     // the scale image is free once its copies (issued above) are done
-                    tc_commit_pair_multicast_e(e, &sm.sfb_empty[gseq % kSfbSlots], 0x3);
+                    tc_commit_pair_multicast_e(e, &sm.sfb_empty[gseq % kSfbSlots], both);
                     ++gseq;
                 }
                 next_stage();
@@ -829,12 +858,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                     next_stage();
                 }
                 if (!aborted) {
-                    tc_commit_pair_multicast_e(e, &sm.tfull[0], 0x3);  // the shared half is complete in both CTAs
+                    tc_commit_pair_multicast_e(e, &sm.tfull[0], both);  // the shared half is complete in both CTAs
                     uint32_t st = stage0;
                     for (int kb = kt; kb < wu.kb1; ++kb) {
                         issue_mmas(wu, kb, st, d_tmem + 128 * (first ^ 1u), idesc128,
                                    (first ^ 1u) * kBoxRows * kAtomBytes, 4 * (first ^ 1u));
-                        tc_commit_pair_multicast_e(e, &sm.empty[st], 0x3);
+                        tc_commit_pair_multicast_e(e, &sm.empty[st], both);
                         if (++st == kStages) st = 0;
                     }
                 }
@@ -843,7 +872,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
                 if (lane == 0) record_timeout(sm, p.status);
                 break;
             }
-            tc_commit_pair_multicast_e(e, &sm.tfull[kTail > 0 ? 1 + (local & 1) : buf], 0x3);  // accumulator complete in both CTAs
+            tc_commit_pair_multicast_e(e, &sm.tfull[kTail > 0 ? 1 + (local & 1) : buf], both);  // accumulator complete in both CTAs
         }
         // All MMAs and copies issued by this warp complete before teardown.
         if (e) {
@@ -860,14 +889,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
         // row n0 + 32j + l -- into two 512-byte tcgen05.cp images.  Warps 2
         // and 3 take alternate groups, so the L2 round trip of one group's
         // loads overlaps the next.
-        const uint32_t sfb_full0 = mapa_shared(smem_u32(&sm.sfb_full[0]), 0);  // the even CTA's
+        const uint32_t sfb_full0 = mapa_shared(smem_u32(&sm.sfb_full[0]), even);  // the even CTA's
         const uint32_t *sfb_words = reinterpret_cast<const uint32_t *>(p.sfb);
         const uint32_t mine = static_cast<uint32_t>(warp - 2);
         uint32_t gseq = 0;
         bool aborted = false;
         PairUnits units(p, pair, num_pairs);
         for (int u = units.next(); u >= 0 && !aborted; u = units.next()) {
-            const WorkUnit wu = work_unit<BN>(p, u);
+            const WorkUnit wu = unit(u);
             for (int kb = wu.kb0; kb < wu.kb1; kb += kStagesPerGroup, ++gseq) {
                 if ((gseq & 1u) != mine) continue;
                 const uint32_t slot = gseq % kSfbSlots;
@@ -914,13 +943,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
         float sab = 1.0f;
         if constexpr (KIND == kGemmFP8Tensor) sab = __fmul_rn(*p.sia, *p.sib);
         uint8_t *stage_buf = sm.epi[q];
-        const uint32_t tempty0 = mapa_shared(smem_u32(&sm.tempty[0]), 0);  // the even CTA's
+        const uint32_t tempty0 = mapa_shared(smem_u32(&sm.tempty[0]), even);  // the even CTA's
         int local = 0;
         uint32_t pieces = 0;  // BF16 output: 32-column pieces stored, alternating staging halves
         PairUnits units(p, pair, num_pairs);
         for (int u = units.next(), un = 0; u >= 0; u = kEarlyLeave ? un : units.next(), ++local) {
             if constexpr (kEarlyLeave) un = units.next();
-            const WorkUnit wu = work_unit<BN>(p, u);
+            const WorkUnit wu = unit(u);
             const int m0 = wu.m0 + kBM * static_cast<int>(rank), n0 = wu.n0;  // this CTA's rows
             const int buf = local % kAccBufs;
             const uint32_t acc_phase = static_cast<uint32_t>(local / kAccBufs) & 1u;
@@ -944,7 +973,82 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
             const int h_first = kShifted ? ((local & 1) ? 0 : 1) : 0;
             constexpr int kHalves = (BN + 127) / 128;
             constexpr int kReleaseAt = kShifted ? 0 : kHalves - 1;
-            if constexpr (OUT_F32) {
+            if constexpr (S > 1) {
+                // one unit: 128 / S columns to each pair of the cluster, then the sum of this CTA's own
+                constexpr int W = 128 / S;
+                const int lr = 32 * q + lane;  // the CTA's row
+                uint32_t own[W];
+#pragma unroll
+                for (int t = 0; t < S; ++t) {
+                    uint32_t v[W / 32][32];
+#pragma unroll
+                    for (int c = 0; c < W / 32; ++c) tmem_ld_32x32b_x32(t_row + W * t + 32 * c, v[c]);
+                    tmem_ld_wait();
+                    if (t == part) {
+#pragma unroll
+                        for (int i = 0; i < W; ++i) own[i] = v[i / 32][i % 32];
+                    } else {
+                        const uint8_t *slot = sm.split.part[part < t ? part : part - 1] + lr * W * 4;
+                        const uint32_t to = mapa_shared(smem_u32(slot), static_cast<uint32_t>(2 * t) + rank);
+#pragma unroll
+                        for (int i = 0; i < W / 4; ++i)
+                            st_cluster_v4(to + 16 * (i ^ (lr & 7)), &v[i / 8][4 * (i % 8)]);
+                    }
+                }
+                leave();
+                cluster_wait();  // every pair's slices have arrived
+                met = true;
+#pragma unroll
+                for (int c = 0; c < W / 32; ++c) {
+                    const int col = n0 + W * part + 32 * c;
+                    if (col >= n_out) break;
+                    float a[32];
+#pragma unroll
+                    for (int t = 0; t < S; ++t) {  // in pair order
+                        const uint8_t *from = sm.split.part[t < part ? t : (t > part ? t - 1 : 0)] + lr * W * 4;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const uint4 x = *reinterpret_cast<const uint4 *>(from + 16 * ((8 * c + i) ^ (lr & 7)));
+                            const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const float b = __uint_as_float(t == part ? own[32 * c + 4 * i + k] : xs[k]);
+                                a[4 * i + k] = t == 0 ? b : a[4 * i + k] + b;
+                            }
+                        }
+                    }
+                    if (e) bulk_wait_group_read0();
+                    __syncwarp();
+                    if constexpr (OUT_F32) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            float f[4];
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                f[k] = KIND == kGemmFP8Tensor ? __fmul_rn(a[4 * i + k], sab) : a[4 * i + k];
+                            *reinterpret_cast<float4 *>(stage_buf + 128 * lane + 16 * (i ^ (lane & 7))) =
+                                make_float4(f[0], f[1], f[2], f[3]);
+                        }
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            uint32_t w[4];
+                            pack_bf16x8<KIND>(reinterpret_cast<const uint32_t *>(&a[8 * i]), sab, w);
+                            *reinterpret_cast<uint4 *>(stage_buf + 64 * lane + 16 * (i ^ ((lane >> 1) & 3))) =
+                                make_uint4(w[0], w[1], w[2], w[3]);
+                        }
+                    }
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (e) {
+                        if constexpr (OUT_F32)
+                            tma_reduce_add_2d(md, stage_buf, col, m0 + 32 * q);
+                        else
+                            tma_store_2d(md, stage_buf, col, m0 + 32 * q);
+                        bulk_commit_group();
+                    }
+                }
+            } else if constexpr (OUT_F32) {
                 // FP32 tile: chunks of 32 columns (128 bytes per row), stored
                 // as a split partial or added to D.  Bound by the reduce-adds
                 // (8 bytes of main-grad traffic per element), so the next
@@ -1076,7 +1180,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(gemm_threads<OUT>(),
         tmem_dealloc_pair(tmem, kTmemCols);
     }
     __syncthreads();
-    if (warp != 1) cluster_wait();
+    if (warp != 1 && !met) cluster_wait();
 }
 
 // Split-K reduction: out[i] = bf16(sum_s ws[s][i]) in fixed order s = 0, 1, ...
@@ -1214,6 +1318,28 @@ int choose_grouped_tile_n(int64_t M, int64_t N, int64_t K) {
     return best;
 }
 
+// Pairs per cluster (4 or 2) that share each 128-wide tile of a GEMM that would
+// split its reduction into `splits` chunks through memory, or 1 to split it
+// there.  The cluster form needs a cluster of eight or four CTAs per tile at
+// once (15 and 36 of them fit) and two stages a pair, and saves the FP32
+// partials' way through memory and the reduction kernel, about 6000 cycles;
+// its exchange costs about 2000 (eight calls with rotating operands in a graph,
+// us a call, through memory and in clusters: [128, 256] x 4096 11.5 and 8.4,
+// [256, 1536] x 4096 11.9 and 9.6, x 8960 14.2 and 12.4, [512, 2048] x 6144
+// 14.7 and 12.0, [768, 1536] x 8960 17.0 and 15.0).
+int cluster_split(int64_t M, int64_t N, int64_t K, int splits) {
+    const int64_t stages = (K + 255) / 256, tiles = pair_tiles(M, N, 128);
+    const int64_t kblocks = (K + 127) / 128, chunk = ((kblocks + splits - 1) / splits + 3) / 4 * 4;
+    const int64_t rounds = (pair_tiles(M, N, 256) * splits + kSplitRefPairs - 1) / kSplitRefPairs;
+    const int64_t through_memory = rounds * (chunk * 4 * kTileCosts[0].per_mma + kTileCosts[0].per_tile) + 6000;
+    for (const int s : {4, 2}) {
+        if (tiles > (s == 4 ? 15 : 36) || stages < 2 * s) continue;
+        const int64_t cost = (stages + s - 1) / s * 8 * kTileCosts[2].per_mma + kTileCosts[2].per_tile + 2000;
+        return cost < through_memory ? s : 1;
+    }
+    return 1;
+}
+
 int64_t splitk_rows_per_chunk(int64_t M) { return (M + kPairM - 1) / kPairM * kPairM; }
 
 size_t splitk_workspace_bytes(int64_t M, int64_t N, int64_t K, bool bf16) {
@@ -1308,6 +1434,18 @@ static cudaError_t launch_params(const GemmParams &p, const GemmArgs &g, const G
                       OUT == kGemmOutF32Partial ? m.ws : m.d, m.sfa, m.sfb, m1.a, m1.b, m1.d, m1.sfa, m1.sfb, p);
 }
 
+// S pairs per tile, one cluster per tile.
+template <int KIND, int OUT, int S>
+static cudaError_t launch_cluster(const GemmArgs &g, const GemmMaps &m, cudaStream_t s) {
+    auto kern = gemm_tn_kernel<KIND, OUT, 128, S>;
+    const size_t smem = sizeof(GemmSmem<128, false, S>) + 1024;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+    const GemmParams p = make_params<KIND, OUT, 128>(g, 1);
+    return launch_pdl(kern, dim3(2 * S * p.num_tiles), dim3(kThreads), smem, s, m.a, m.b, m.d, m.sfa, m.sfb, m.a, m.b,
+                      m.d, m.sfa, m.sfb, p);
+}
+
 template <int KIND, int OUT, int BN>
 static cudaError_t launch_kind(const GemmArgs &g, const GemmMaps &m, int splits, cudaStream_t s) {
     return launch_params<KIND, OUT, BN>(make_params<KIND, OUT, BN>(g, splits), g, m, m, s);
@@ -1333,6 +1471,12 @@ static cudaError_t launch_split_or_not(const GemmArgs &g, const GemmMaps &m, cud
             if (g.tile_n == 224) return launch_kind<KIND, kGemmOutBF16, 224>(g, m, 1, s);
         return launch_width<KIND, kGemmOutBF16>(g, m, s);
     }
+    if (g.cluster == 2)
+        return g.accumulate_f32 ? launch_cluster<KIND, kGemmOutF32Add, 2>(g, m, s)
+                                : launch_cluster<KIND, kGemmOutBF16, 2>(g, m, s);
+    if (g.cluster == 4)
+        return g.accumulate_f32 ? launch_cluster<KIND, kGemmOutF32Add, 4>(g, m, s)
+                                : launch_cluster<KIND, kGemmOutBF16, 4>(g, m, s);
     cudaError_t e = launch_kind<KIND, kGemmOutF32Partial, 256>(g, m, g.splits, s);
     if (e != cudaSuccess) return e;
     const int64_t n4 = g.M * g.N / 4;

@@ -149,6 +149,7 @@ struct GemmArgs {
     // split reduction (FP8 kinds only): splits > 1 needs `workspace` of
     // splitk_workspace_bytes(M, N, K) bytes; `out` is D (bf16)
     int splits;
+    int cluster;                 // splits > 1: pairs of a cluster that share the reduction on chip (2 or 4), or 1
     void *workspace;
     void *out;
     // out is an FP32 main-grad [M, N] that receives out += A * B^T (block
@@ -197,6 +198,7 @@ puro_status_t fp8_gemm_validate(const puro_fp8_tensor_t *a, const puro_fp8_tenso
 // then needs.  Host-only, shape-only (plans for 152 SMs).
 int choose_splits(int64_t M, int64_t N, int64_t K, bool bf16);
 size_t splitk_workspace_bytes(int64_t M, int64_t N, int64_t K, bool bf16);
+int cluster_split(int64_t M, int64_t N, int64_t K, int splits);  // see GemmArgs::cluster
 int64_t splitk_rows_per_chunk(int64_t M);  // M rounded up to a whole 256-row pair tile
 // Whether a linear's Dgrad (dX [M, K], reduction N) and Wgrad (dW [N, K],
 // reduction M) are modelled faster as one grouped launch (balanced

@@ -218,7 +218,14 @@ PURO_DEV uint32_t cluster_ctarank() {
     return r;
 }
 
-// All threads of both CTAs of the cluster (release / acquire).
+// Store to shared memory of a cluster CTA (16-byte aligned address from mapa_shared).
+PURO_DEV void st_cluster_v4(uint32_t addr, const uint32_t *v) {
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                 "r"(v[3])
+                 : "memory");
+}
+
+// All threads of all CTAs of the cluster (release / acquire).
 PURO_DEV void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }

@@ -341,6 +341,36 @@ def test_block_gemm_tail_halves(K, main_grad):
     check_gemm_every_tile(out, A, B, np.random.default_rng(8300 + K), "tail halves")
 
 
+# A reduction split on chip: four pairs of a cluster per 128-wide tile (up to 15
+# tiles) or two (up to 36), whole and ragged extents, the last part shorter.
+@pytest.mark.parametrize("scaling,M,N,K", [(P.SCALE_BLOCK, 128, 128, 4096), (P.SCALE_BLOCK, 256, 1536, 8960),
+                                           (P.SCALE_BLOCK, 512, 1664, 4224), (P.SCALE_TENSOR, 272, 400, 8208),
+                                           (P.SCALE_TENSOR, 528, 1424, 6160)])
+@pytest.mark.parametrize("main_grad", [False, True])
+def test_gemm_reduction_split_in_a_cluster(scaling, M, N, K, main_grad):
+    assert P.puro_fp8_workspace_size(M, N, K) > 0
+    x, w, _ = _inputs(M, N, K, 8400 + M + N + K, t3=True)
+    xq, wq = (P.quantize(t, P.E4M3, scaling, P.ROLE_ACT) for t in (x, w))
+    ws = torch.full((P.puro_fp8_workspace_size(M, N, K),), 0xFF, dtype=torch.uint8, device=DEV)
+    start = W.normal_f32((M, N), 1.0, DEV, 8450) if main_grad else None
+    outs = []
+    for _ in range(2):
+        out = start.clone() if main_grad else torch.empty((M, N), dtype=torch.bfloat16, device=DEV)
+        status = torch.zeros(1, dtype=torch.int32, device=DEV)
+        call = P.puro_fp8_linear_wgrad_main_grad if main_grad else P.puro_fp8_linear_fprop
+        call(xq.rowwise, wq.rowwise, out, ws, status)
+        torch.cuda.synchronize()
+        assert P.puro_fp8_get_status(status) == 0
+        outs.append(out)
+    assert torch.equal(outs[0], outs[1])  # the order of the sum is fixed
+    if scaling == P.SCALE_BLOCK:
+        A, B = (O.dequant_rows_1x128(*par_quantize_rows_1x128(bits(t), P.E4M3), P.E4M3) for t in (x, w))
+        ref = O.gemm_tn(A, B, 8)
+    else:
+        ref = oracle_linear(x, w, torch.zeros((M, N), dtype=torch.bfloat16, device=DEV), scaling)["y"]
+    assert_close(outs[0].double() - start.double() if main_grad else outs[0], ref, "split in a cluster")
+
+
 # --------------------------------------------------------------------------
 # Several tiles per CTA pair.  The persistent grid holds at most 76 pairs on
 # GB300 (152 SMs), so outputs of 256 or more 256-wide pair tiles make every
