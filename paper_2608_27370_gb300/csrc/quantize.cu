@@ -395,18 +395,24 @@ PURO_DEV void tile_codes_to_stage(QuantSmem &sm, const uint2 (&v)[8], int br, in
     if constexpr (HAS_T) stage_transposed_8x4(sm.qt_stage, rw, br, bc);
 }
 
-// Row and column block of a persistent CTA's tiles t, t + step, t + 2 step,
-// ... in a grid of tiles_n column blocks, advanced without a division.
+// Row and column block of a persistent CTA's tiles t, t - step, t - 2 step,
+// ... in a grid of tiles_n column blocks, stepped without a division.  From
+// the last tile backwards: the amax, rstd or GEMM pass before wrote or read the
+// tensor forwards, so its end is what L2 still holds, and the GEMM behind
+// starts with the codes written last.  Against forwards: a block-scaled linear
+// of [8192, 2048] x 2048 115.3 -> 114.6 us, [32768, 1536] x 17920
+// 2116 -> 2107 us, an MLP forward of [8192, 2048], 6144 wide, 276.8 -> 275.2 us;
+// tensors that fit in L2 whole: the same.
 struct TileWalk {
     int r, c, dr, dc, n;
     PURO_DEV TileWalk(int t, int step, int tiles_n)
         : r(t / tiles_n), c(t % tiles_n), dr(step / tiles_n), dc(step % tiles_n), n(tiles_n) {}
     PURO_DEV void advance() {
-        r += dr;
-        c += dc;
-        if (c >= n) {
-            c -= n;
-            ++r;
+        r -= dr;
+        c -= dc;
+        if (c < 0) {
+            c += n;
+            --r;
         }
     }
 };
@@ -472,7 +478,7 @@ __global__ void __launch_bounds__(kQThreads, 2)
         tma_load_2d(sm.in[b], &tm_x, &sm.full[b], t.c * kQT, t.r * kQT);
     };
     int tile = blockIdx.x;
-    TileWalk cur(tile, gridDim.x, tiles_n), nxt = cur;
+    TileWalk cur(ntiles - 1 - tile, gridDim.x, tiles_n), nxt = cur;
     nxt.advance();
     if (tid == 0 && tile < ntiles) issue_load(cur, 0);
     for (int it = 0; tile < ntiles; ++it, tile += gridDim.x, cur = nxt, nxt.advance()) {
@@ -661,7 +667,7 @@ __global__ void __launch_bounds__(kQAThreads, 2)
     };
     int tile = blockIdx.x;
     const int step = gridDim.x;
-    TileWalk cur(tile, step, tiles_n), nxt = cur;  // this tile and the CTA's next one
+    TileWalk cur(ntiles - 1 - tile, step, tiles_n), nxt = cur;  // this tile and the CTA's next one
     nxt.advance();
     // RMSNorm: the kernel before this one on the stream is the rstd pass over
     // the same h, whose CTAs all passed their own pdl_wait before this grid
