@@ -78,11 +78,16 @@ __device__ __forceinline__ int matrix_of(const MuonhGroup &g, int b) {
     return lo;
 }
 
-// Per-CTA partial sums {S_ww, S_wu, S_uu} of one chunk.
+// Per-CTA partial sums {S_ww, S_wu, S_uu} of one chunk; the last chunk first, so
+// that the update, which goes forwards, finds in L2 what was read last.  The
+// step is bound by HBM (two passes).  Against both passes forwards, us: one
+// layer of Qwen2-1.5B 181.6 -> 171.7, of Qwen3-1.7B 196.1 -> 183.8; 7 layers
+// 1116 -> 1096, 28 layers 4751 -> 4662 (turning the update round instead:
+// 180.3, 188.0, 1113, 4739).
 __global__ void __launch_bounds__(kMuonhThreads) muonh_reduce_kernel(const __grid_constant__ MuonhGroup g) {
     pdl_wait();
     pdl_launch_dependents();
-    const int b = blockIdx.x;
+    const int b = static_cast<int>(gridDim.x - 1 - blockIdx.x);
     const int m = matrix_of(g, b);
     const int64_t c4 = g.chunk4[m];
     const int64_t lo = static_cast<int64_t>(b - g.block_start[m]) * c4;
