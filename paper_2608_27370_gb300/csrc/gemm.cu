@@ -977,24 +977,39 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
                 // one unit: 128 / S columns to each pair of the cluster, then the sum of this CTA's own
                 constexpr int W = 128 / S;
                 const int lr = 32 * q + lane;  // the CTA's row
-                uint32_t own[W];
 #pragma unroll
-                for (int t = 0; t < S; ++t) {
+                for (int i = 1; i < S; ++i) {
+                    const int t = (part + i) & (S - 1);
+                    const uint32_t slot = smem_u32(sm.split.part[part < t ? part : part - 1] + 32 * q * W * 4);
+                    const uint32_t to = mapa_shared(slot, static_cast<uint32_t>(2 * t) + rank);
                     uint32_t v[W / 32][32];
 #pragma unroll
                     for (int c = 0; c < W / 32; ++c) tmem_ld_32x32b_x32(t_row + W * t + 32 * c, v[c]);
                     tmem_ld_wait();
-                    if (t == part) {
 #pragma unroll
-                        for (int i = 0; i < W; ++i) own[i] = v[i / 32][i % 32];
-                    } else {
-                        const uint8_t *slot = sm.split.part[part < t ? part : part - 1] + lr * W * 4;
-                        const uint32_t to = mapa_shared(smem_u32(slot), static_cast<uint32_t>(2 * t) + rank);
+                    for (int c = 0; c < W / 32; ++c) {
+                        // Through the staging tile, so that eight lanes store 128
+                        // bytes of a row: a lane's own row in 16-byte stores took
+                        // 3.3 us instead of 1.2 for S = 4 ([256, 1536] x 8960 12.3
+                        // -> 10.1 us, [512, 2048] x 6144 at S = 2 11.9 -> 11.1).
 #pragma unroll
-                        for (int i = 0; i < W / 4; ++i)
-                            st_cluster_v4(to + 16 * (i ^ (lr & 7)), &v[i / 8][4 * (i % 8)]);
+                        for (int k = 0; k < 8; ++k)
+                            *reinterpret_cast<uint4 *>(stage_buf + 128 * lane + 16 * (k ^ (lane & 7))) =
+                                make_uint4(v[c][4 * k], v[c][4 * k + 1], v[c][4 * k + 2], v[c][4 * k + 3]);
+                        __syncwarp();
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const int row = 4 * k + lane / 8, at = 16 * (lane % 8);
+                            st_cluster_v4(to + row * W * 4 + 128 * c + at,
+                                          *reinterpret_cast<const uint4 *>(stage_buf + 128 * row + at));
+                        }
+                        __syncwarp();
                     }
                 }
+                uint32_t own[W / 32][32];
+#pragma unroll
+                for (int c = 0; c < W / 32; ++c) tmem_ld_32x32b_x32(t_row + W * part + 32 * c, own[c]);
+                tmem_ld_wait();
                 leave();
                 cluster_wait();  // every pair's slices have arrived
                 met = true;
@@ -1012,7 +1027,7 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
                             const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
                             for (int k = 0; k < 4; ++k) {
-                                const float b = __uint_as_float(t == part ? own[32 * c + 4 * i + k] : xs[k]);
+                                const float b = __uint_as_float(t == part ? own[c][4 * i + k] : xs[k]);
                                 a[4 * i + k] = t == 0 ? b : a[4 * i + k] + b;
                             }
                         }
@@ -1324,9 +1339,9 @@ int choose_grouped_tile_n(int64_t M, int64_t N, int64_t K) {
 // once (15 and 36 of them fit) and two stages a pair, and saves the FP32
 // partials' way through memory and the reduction kernel, about 6000 cycles;
 // its exchange costs about 2000 (eight calls with rotating operands in a graph,
-// us a call, through memory and in clusters: [128, 256] x 4096 11.5 and 8.4,
-// [256, 1536] x 4096 11.9 and 9.6, x 8960 14.2 and 12.4, [512, 2048] x 6144
-// 14.7 and 12.0, [768, 1536] x 8960 17.0 and 15.0).
+// us a call, through memory and in clusters: [128, 256] x 4096 11.5 and 6.4,
+// [256, 1536] x 4096 11.9 and 7.0, x 8960 14.2 and 10.1, [512, 2048] x 6144
+// 14.7 and 11.1, [768, 1536] x 8960 17.0 and 14.2).
 int cluster_split(int64_t M, int64_t N, int64_t K, int splits) {
     const int64_t stages = (K + 255) / 256, tiles = pair_tiles(M, N, 128);
     const int64_t kblocks = (K + 127) / 128, chunk = ((kblocks + splits - 1) / splits + 3) / 4 * 4;

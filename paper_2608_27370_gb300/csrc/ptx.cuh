@@ -219,9 +219,8 @@ PURO_DEV uint32_t cluster_ctarank() {
 }
 
 // Store to shared memory of a cluster CTA (16-byte aligned address from mapa_shared).
-PURO_DEV void st_cluster_v4(uint32_t addr, const uint32_t *v) {
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]),
-                 "r"(v[3])
+PURO_DEV void st_cluster_v4(uint32_t addr, const uint4 &v) {
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
                  : "memory");
 }
 
