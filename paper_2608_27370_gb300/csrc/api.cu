@@ -160,6 +160,7 @@ puro_status_t prepare_fp8_gemm(const puro_fp8_tensor_t *a, const puro_fp8_tensor
     g.N = N;
     g.K = K;
     g.tile_n = tile_n;
+    g.b = static_cast<const uint8_t *>(b->data);
     if (block) {
         if (!make_scale_map(&m.sfa, a->scale, M, K) || !make_scale_map(&m.sfb, b->scale, N, K)) return PURO_ERR_CUDA;
         g.sfb = static_cast<const uint8_t *>(b->scale);

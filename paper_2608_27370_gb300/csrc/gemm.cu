@@ -69,6 +69,8 @@ constexpr int kTmemCols = 512;
 constexpr int kSfColsPerSet = 12;  // 4 for A (128 rows) + 8 for B (up to 256 rows)
 constexpr int kSfSets = 2;         // double-buffered across groups of four k-blocks
 constexpr int kTailBlocks = 3;     // k-blocks of a shifted tile issued as halves
+constexpr uint32_t kPrefetchNs = 100;  // pause between the k-blocks of B a waiting CTA prefetches
+constexpr int64_t kPrefetchBytes = 8 << 20;  // a smaller B is not worth the prologue's time (0.1 us)
 constexpr uint32_t kAllocBarrier = 7, kLeaveBarrier = 8;  // named barriers (the quantising epilogue uses 1..6)
 constexpr int kSfbSlots = 4;       // BN = 224: ring of helper-built B scale images
 constexpr uint64_t kDrainTimeoutNs = 2000000000ull;
@@ -139,6 +141,7 @@ struct GemmSmem {
     uint64_t drain;
     uint32_t tmem_base;
     volatile int abort_flag;
+    volatile int started;  // the producer is past its wait for the kernel before
     std::conditional_t<QOUT, QuantEpiSmem, NoQuantEpiSmem> qe;
     std::conditional_t<(S > 1), SplitSmem<S>, NoSplitSmem> split;
 };
@@ -173,6 +176,7 @@ struct GemmParams {
     // Grouped launch: short (second-problem) units the pairs with one long
     // unit fewer take first (see PairUnits); 0: plain round-robin.
     int lead;
+    const uint8_t *b;  // B (rows of K bytes) where it is prefetched, or null
 };
 
 // Instruction descriptors (tcgen05.mma), both operands K-major, M = 256
@@ -617,6 +621,7 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
         }
         mbar_init(&sm.drain, 1);
         sm.abort_flag = 0;
+        sm.started = 0;
         fence_mbarrier_init();
         tma_prefetch_desc(&tm_a);
         tma_prefetch_desc(&tm_b);
@@ -646,8 +651,30 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
         tc_fence_after_sync();
     }
     cluster_wait();
+    // A launch of one unit a pair is latency-bound and a B of some size is often
+    // a weight that has left L2: while the kernel before runs, the epilogue's
+    // warps prefetch it (into L2 only, so it may still be being written), a
+    // k-block at a time until the producer starts.  Unpaced, the flood delayed
+    // the first k-blocks where there was nothing to wait for (9.6 -> 10.3 us on
+    // the first shape below).  With the quantiser of A ahead, ten and more weights
+    // in turn, us both: [256, 17920] x 1536 14.1 -> 13.1, [256, 12288] x 2048
+    // 13.8 -> 13.2, [256, 1536] x 8960 14.4 -> 14.1, [128, 6144] x 2048 10.2 ->
+    // 10.0; one weight that stays in L2 12.5, 12.5, 13.1 -> 13.0, 9.4 -> 9.5.
+    if (p.b && warp >= 4 && p.num_units <= num_pairs) {
+        const WorkUnit wu = unit(pair);
+        const int row = wu.n0 + kBNHalf * static_cast<int>(rank) + static_cast<int>(threadIdx.x) - 128;
+        if (wu.m0 == 0 && static_cast<int>(threadIdx.x) - 128 < kBNHalf && row < p.N) {
+            const uint8_t *b = p.b + static_cast<int64_t>(row) * p.K;
+            const int k1 = min(p.K, wu.kb1 * kBK);
+            for (int k = wu.kb0 * kBK; k < k1 && !sm.started; k += 128) {
+                prefetch_l2(b + k);
+                __nanosleep(kPrefetchNs);
+            }
+        }
+    }
     pdl_wait();  // the set-up above overlaps the previous kernel's tail
     pdl_launch_dependents();
+    if (threadIdx.x == 0) sm.started = 1;
     const uint32_t tmem = warp != 0 ? sm.tmem_base : 0u;
     // Arrive at the closing cluster barrier: this warp is done with tensor
     // memory and the peer's barriers.
@@ -1418,6 +1445,7 @@ static GemmParams make_params(const GemmArgs &g, int splits) {
         p.idesc = idesc_mx(static_cast<uint32_t>(g.a_fmt), static_cast<uint32_t>(g.b_fmt), BN);
     p.kgroups = static_cast<int>((g.K / 128 + 3) / 4);
     p.sfb = g.sfb;
+    p.b = g.N * g.K >= kPrefetchBytes ? g.b : nullptr;
     p.sia = g.sia;
     p.sib = g.sib;
     p.status = g.status;
@@ -1514,6 +1542,7 @@ template <int BN>
 static cudaError_t launch_grouped_width(const GemmArgs &g0, const GemmMaps &m0, const GemmArgs &g1,
                                         const GemmMaps &m1, cudaStream_t s) {
     GemmParams p = make_params<kGemmFP8Block, kGemmOutBF16, BN>(g0, 1);
+    p.b = nullptr;
     const GemmParams q = make_params<kGemmFP8Block, kGemmOutBF16, BN>(g1, 1);
     p.units0 = p.num_units;
     p.N1 = q.N;

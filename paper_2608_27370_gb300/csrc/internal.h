@@ -140,6 +140,7 @@ struct GemmArgs {
     int tile_n;                  // 256, 192 or 128 (see choose_tile_n), or 224 (block kind, BF16 out, forced); split: 256
     // kGemmFP8Block: scale vectors of B (the 224-wide form gathers them
     // itself; the others load them through GemmMaps::sfb).
+    const uint8_t *b;            // FP8 kinds: B's codes
     const uint8_t *sfb;
     // kGemmFP8Tensor: dequantisation factors of A and B.
     const float *sia, *sib;

@@ -270,6 +270,9 @@ PURO_DEV void tma_load_2d_pair_e(uint32_t e, void *dst, const CUtensorMap *map, 
         : "memory");
 }
 
+// The 128-byte line at p into L2 (a hint: nothing waits for it).
+PURO_DEV void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 PURO_DEV void tmem_alloc_pair(uint32_t *dst_smem, uint32_t ncols) {  // one warp in each CTA of the pair
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),
                  "r"(ncols)

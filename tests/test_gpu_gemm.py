@@ -341,6 +341,32 @@ def test_block_gemm_tail_halves(K, main_grad):
     check_gemm_every_tile(out, A, B, np.random.default_rng(8300 + K), "tail halves")
 
 
+# A launch of one tile a pair prefetches a B of 8 MB or more while the kernel before still runs:
+# here that kernel writes B, over the previous values.
+@pytest.mark.parametrize("M,N,K", [(128, 17920, 1536), (256, 4096, 2048), (256, 1536, 8960)])
+def test_gemm_right_behind_the_quantiser_of_b(M, N, K):
+    x, _, _ = _inputs(M, 128, K, 8700 + N, t3=True)
+    xq = P.quantize(x, P.E4M3).rowwise
+    ws = torch.empty(max(16, P.puro_fp8_workspace_size(M, N, K)), dtype=torch.uint8, device=DEV)
+    weights = [W.normal_bf16((N, K), 0.02, DEV, 8710 + i) for i in range(3)]
+    wq = P.quantize(weights[0], P.E4M3, P.SCALE_BLOCK, P.ROLE_WEIGHT)
+
+    def outputs(sync):
+        ys = []
+        for w in weights:
+            y = torch.empty((M, N), dtype=torch.bfloat16, device=DEV)
+            P.quantize(w, P.E4M3, P.SCALE_BLOCK, P.ROLE_WEIGHT, out=wq)
+            if sync:
+                torch.cuda.synchronize()
+            P.puro_fp8_linear_fprop(xq, wq.rowwise, y, ws)
+            ys.append(y)
+        torch.cuda.synchronize()
+        return ys
+
+    for behind, alone in zip(outputs(False), outputs(True)):
+        assert torch.equal(behind, alone)
+
+
 # A reduction split on chip: four pairs of a cluster per 128-wide tile (up to 15
 # tiles) or two (up to 36), whole and ragged extents, the last part shorter.
 @pytest.mark.parametrize("scaling,M,N,K", [(P.SCALE_BLOCK, 128, 128, 4096), (P.SCALE_BLOCK, 256, 1536, 8960),
