@@ -431,6 +431,10 @@ PURO_DEV uint32_t block_max_8x4(const uint2 (&v)[8]) {
 // 8*(t/32) .. +7 and columns 4*(t%32) .. +3.  The weight kind reduces the
 // block maximum through the warps (one barrier); the per-tensor kind reads
 // its scale from the device amax.
+// Barriers and descriptors are ready before the wait for the kernel ahead and
+// the first tile is in flight before the scale is read: after it, one after the
+// other, amax and cast took 5.2 us instead of 4.8 on [256, 1536], 7.4 instead of
+// 6.9 on [2048, 2048] and 16.5 instead of 15.5 on [4112, 3968].
 template <int FMT, int KIND, bool HAS_T>
 __global__ void __launch_bounds__(kQThreads, 2)
     quant_tile_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_q,
@@ -445,22 +449,6 @@ __global__ void __launch_bounds__(kQThreads, 2)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int br = warp;  // block row: tile rows 8br .. 8br+7
     const int bc = lane;  // block column: tile columns 4bc .. 4bc+3
-    pdl_wait();
-    pdl_launch_dependents();
-
-    // Per-tensor mode: the one scale, from the device amax.
-    float t_mul = 1.0f;
-    if constexpr (KIND == kQuantTensor) {
-        const uint32_t a = *amax_bits & 0xFFFFu;
-        const bool t_nan = a >= 0x7F80u;
-        const float t_scale = tensor_scale<FMT>(a);
-        t_mul = t_nan ? __uint_as_float(0x7FC00000u) : t_scale;
-        if (blockIdx.x == 0 && tid == 0) {
-            const float si = t_nan ? __uint_as_float(0x7FC00000u) : __fdiv_rn(1.0f, t_scale);
-            *scale_f = si;
-            if (scale_t_f) *scale_t_f = si;
-        }
-    }
     if (tid == 0) {
         mbar_init(&sm.full[0], 1);
         mbar_init(&sm.full[1], 1);
@@ -480,7 +468,25 @@ __global__ void __launch_bounds__(kQThreads, 2)
     int tile = blockIdx.x;
     TileWalk cur(ntiles - 1 - tile, gridDim.x, tiles_n), nxt = cur;
     nxt.advance();
+    pdl_wait();  // the set-up above overlaps the kernel before
+    pdl_launch_dependents();
     if (tid == 0 && tile < ntiles) issue_load(cur, 0);
+    bool gave_up = false;  // a zero wait bound is one test right after the load is issued
+    if (KIND == kQuantTensor && tid == 0 && wait_ns == 0 && tile < ntiles) gave_up = !mbar_test_wait(&sm.full[0], 0);
+
+    // Per-tensor mode: the one scale, from the device amax, while the tile streams in.
+    float t_mul = 1.0f;
+    if constexpr (KIND == kQuantTensor) {
+        const uint32_t a = *amax_bits & 0xFFFFu;
+        const bool t_nan = a >= 0x7F80u;
+        const float t_scale = tensor_scale<FMT>(a);
+        t_mul = t_nan ? __uint_as_float(0x7FC00000u) : t_scale;
+        if (blockIdx.x == 0 && tid == 0) {
+            const float si = t_nan ? __uint_as_float(0x7FC00000u) : __fdiv_rn(1.0f, t_scale);
+            *scale_f = si;
+            if (scale_t_f) *scale_t_f = si;
+        }
+    }
     for (int it = 0; tile < ntiles; ++it, tile += gridDim.x, cur = nxt, nxt.advance()) {
         const int buf = it & 1;
         const int64_t r0 = static_cast<int64_t>(cur.r) * kQT;
@@ -496,7 +502,7 @@ __global__ void __launch_bounds__(kQThreads, 2)
         // Every thread waits on the tile's barrier itself, which makes the
         // TMA-written tile visible to it.  A wait that runs out is voted on
         // at the next barrier, where every thread leaves together.
-        const bool landed = tile_landed(&sm.full[buf], static_cast<uint32_t>(it >> 1) & 1u, wait_ns);
+        const bool landed = tile_landed(&sm.full[buf], static_cast<uint32_t>(it >> 1) & 1u, wait_ns) && !gave_up;
         if constexpr (KIND == kQuantTensor) {
             if (__syncthreads_or(!landed)) {  // (S1) staging free
                 if (tid == 0) quant_abort(sm.full, it, tile + static_cast<int>(gridDim.x) < ntiles, status);
@@ -965,15 +971,6 @@ __global__ void __launch_bounds__(kQThreads, 2) quant_weight_group_kernel(const 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int br = warp;  // block row: tile rows 8br .. 8br+7
     const int bc = lane;  // block column: tile columns 4bc .. 4bc+3
-    pdl_wait();
-    pdl_launch_dependents();
-    if (tid == 0) {
-        mbar_init(&sm.full[0], 1);
-        mbar_init(&sm.full[1], 1);
-        fence_mbarrier_init();
-    }
-    __syncthreads();
-
     const int ntiles = g.tile_start[g.count];
     // the weight of tile t, scanning forward from w (tiles only increase)
     auto locate = [&](int t, int w) {
@@ -987,10 +984,19 @@ __global__ void __launch_bounds__(kQThreads, 2) quant_weight_group_kernel(const 
     };
     int tile = blockIdx.x;
     int w = 0;
-    if (tile < ntiles) {
-        w = locate(tile, 0);
-        if (tid == 0) issue_load(tile, w, 0);
+    if (tile < ntiles) w = locate(tile, 0);
+    if (tid == 0) {
+        mbar_init(&sm.full[0], 1);
+        mbar_init(&sm.full[1], 1);
+        fence_mbarrier_init();
+        tma_prefetch_desc(&g.x[w]);
+        tma_prefetch_desc(&g.q[w]);
+        if (HAS_T) tma_prefetch_desc(&g.qt[w]);
     }
+    __syncthreads();
+    pdl_wait();  // the set-up above overlaps the kernel before
+    pdl_launch_dependents();
+    if (tid == 0 && tile < ntiles) issue_load(tile, w, 0);
     for (int it = 0; tile < ntiles; ++it, tile += gridDim.x) {
         w = locate(tile, w);
         const int buf = it & 1;
