@@ -977,14 +977,18 @@ __global__ void __launch_bounds__(kQThreads, 2) quant_weight_group_kernel(const 
         while (t >= g.tile_start[w + 1]) ++w;
         return w;
     };
-    auto issue_load = [&](int t, int w, int b) {
-        const int lt = t - g.tile_start[w];
+    auto column_of = [&](int t, int w) { return (t - g.tile_start[w]) % g.tiles_n[w] * kQT; };
+    auto row_of = [&](int t, int w) { return (t - g.tile_start[w]) / g.tiles_n[w] * kQT; };
+    auto issue_load = [&](int w, int b, int x, int y) {
         mbar_arrive_expect_tx(&sm.full[b], kQT * kQT * 2);
-        tma_load_2d(sm.in[b], &g.x[w], &sm.full[b], (lt % g.tiles_n[w]) * kQT, (lt / g.tiles_n[w]) * kQT);
+        tma_load_2d(sm.in[b], &g.x[w], &sm.full[b], x, y);
     };
     int tile = blockIdx.x;
     int w = 0;
     if (tile < ntiles) w = locate(tile, 0);
+    // divided ahead of the wait (the empty asm keeps it there): [2048, 2048] 4.1 -> 3.9 us
+    int x0 = column_of(tile, w), y0 = row_of(tile, w);
+    asm volatile("" : "+r"(x0), "+r"(y0));
     if (tid == 0) {
         mbar_init(&sm.full[0], 1);
         mbar_init(&sm.full[1], 1);
@@ -996,7 +1000,7 @@ __global__ void __launch_bounds__(kQThreads, 2) quant_weight_group_kernel(const 
     __syncthreads();
     pdl_wait();  // the set-up above overlaps the kernel before
     pdl_launch_dependents();
-    if (tid == 0 && tile < ntiles) issue_load(tile, w, 0);
+    if (tid == 0 && tile < ntiles) issue_load(w, 0, x0, y0);
     for (int it = 0; tile < ntiles; ++it, tile += gridDim.x) {
         w = locate(tile, w);
         const int buf = it & 1;
@@ -1005,7 +1009,10 @@ __global__ void __launch_bounds__(kQThreads, 2) quant_weight_group_kernel(const 
         const int64_t c0 = static_cast<int64_t>(lt % g.tiles_n[w]) * kQT;
         if (tid == 0) {
             const int next = tile + gridDim.x;
-            if (next < ntiles) issue_load(next, locate(next, w), buf ^ 1);  // buffer last read before (S3) of it-1
+            if (next < ntiles) {  // buffer last read before (S3) of it-1
+                const int wn = locate(next, w);
+                issue_load(wn, buf ^ 1, column_of(next, wn), row_of(next, wn));
+            }
         }
         const bool landed = tile_landed(&sm.full[buf], static_cast<uint32_t>(it >> 1) & 1u, g.wait_ns);
 
