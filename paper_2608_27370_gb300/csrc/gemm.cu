@@ -1026,7 +1026,7 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
                         // Through the staging tile, so that eight lanes store 128
                         // bytes of a row: a lane's own row in 16-byte stores took
                         // 3.3 us instead of 1.2 for S = 4 ([256, 1536] x 8960 12.3
-                        // -> 10.1 us, [512, 2048] x 6144 at S = 2 11.9 -> 11.1).
+                        // -> 10.1 us).
 #pragma unroll
                         for (int k = 0; k < 8; ++k)
                             *reinterpret_cast<uint4 *>(stage_buf + 128 * lane + 16 * (k ^ (lane & 7))) =
@@ -1371,19 +1371,19 @@ int choose_grouped_tile_n(int64_t M, int64_t N, int64_t K) {
 // Pairs per cluster (4 or 2) that share each 128-wide tile of a GEMM that would
 // split its reduction into `splits` chunks through memory, or 1 to split it
 // there.  The cluster form needs a cluster of eight or four CTAs per tile at
-// once (15 and 36 of them fit) and two stages a pair, and saves the FP32
+// once (15 and 36 of them fit), two stages a pair and, since a longer chain of
+// FP32 additions is less exact, no fewer parts than chunks, and saves the FP32
 // partials' way through memory and the reduction kernel, about 6000 cycles;
 // its exchange costs about 2000 (eight calls with rotating operands in a graph,
 // us a call, through memory and in clusters: [128, 256] x 4096 11.5 and 6.4,
-// [256, 1536] x 4096 11.9 and 7.0, x 8960 14.2 and 10.1, [512, 2048] x 6144
-// 14.7 and 11.1, [768, 1536] x 8960 17.0 and 14.2).
+// [256, 1536] x 4096 11.9 and 7.0, x 8960 14.2 and 10.1).
 int cluster_split(int64_t M, int64_t N, int64_t K, int splits) {
     const int64_t stages = (K + 255) / 256, tiles = pair_tiles(M, N, 128);
     const int64_t kblocks = (K + 127) / 128, chunk = ((kblocks + splits - 1) / splits + 3) / 4 * 4;
     const int64_t rounds = (pair_tiles(M, N, 256) * splits + kSplitRefPairs - 1) / kSplitRefPairs;
     const int64_t through_memory = rounds * (chunk * 4 * kTileCosts[0].per_mma + kTileCosts[0].per_tile) + 6000;
     for (const int s : {4, 2}) {
-        if (tiles > (s == 4 ? 15 : 36) || stages < 2 * s) continue;
+        if (s < splits || tiles > (s == 4 ? 15 : 36) || stages < 2 * s) continue;
         const int64_t cost = (stages + s - 1) / s * 8 * kTileCosts[2].per_mma + kTileCosts[2].per_tile + 2000;
         return cost < through_memory ? s : 1;
     }
