@@ -127,9 +127,9 @@ _native = None
 
 
 def _load_native():
-    """The native marshalling module, built and linked against the library at LIB_PATH."""
+    """The native marshalling module, calling the library that load_library() returns."""
     global _native
-    load_library()
+    lib = load_library()
     if not os.path.exists(_build.NATIVE):
         raise RuntimeError(f"{_build.NATIVE} not found: build it with "
                            "`python -c 'import __graft_entry__ as g; g.build()'`")
@@ -138,6 +138,7 @@ def _load_native():
     module = importlib.util.module_from_spec(importlib.util.spec_from_loader(name, loader))
     loader.exec_module(module)
     module.set_operand_type(FP8Operand)
+    module.set_library({n: ctypes.cast(getattr(lib, n), ctypes.c_void_p).value for n in _SIGNATURES})
     _native = module
     return module
 

@@ -3,8 +3,8 @@
 Five translation units are compiled in parallel and linked into one shared
 object with the CUDA runtime linked statically, so the library loads on a
 machine without a GPU driver (only the first CUDA call needs one).  Beside it
-the Python binding's native marshalling module _native.so is compiled against
-the installed torch's headers and linked against the library.
+the Python binding's native marshalling module _native.so is compiled and
+linked against the installed torch (the library's entry points are handed to it).
 """
 from __future__ import annotations
 
@@ -96,8 +96,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
     libs = os.path.join(os.path.dirname(torch.__file__), "lib")
     tmp = NATIVE + ".tmp.%d" % os.getpid()
-    cmd = ["g++", "-shared", "-o", tmp, binding_obj, "-L", PKG, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN",
-           "-L", libs, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    cmd = ["g++", "-shared", "-o", tmp, binding_obj, "-L", libs, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"link of the binding failed:\n{r.stdout}\n{r.stderr}")

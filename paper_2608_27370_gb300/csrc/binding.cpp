@@ -24,6 +24,32 @@ namespace {
 
 PyObject *operand_type = nullptr;  // the binding's FP8Operand class
 
+// The library's entry points, handed over by the binding (set_library): the
+// same library its ctypes calls go to, also where a process holds two copies of
+// the package.  Linked by name, the second copy's module got the first one's.
+#define PURO_ENTRIES(X)                \
+    X(puro_fp8_amax)                   \
+    X(puro_fp8_quantize)               \
+    X(puro_fp8_quantize_rmsnorm)       \
+    X(puro_fp8_quantize_swiglu)        \
+    X(puro_fp8_quantize_weights)       \
+    X(puro_fp8_linear_fprop)           \
+    X(puro_fp8_linear_dgrad)           \
+    X(puro_fp8_linear_wgrad)           \
+    X(puro_fp8_linear_wgrad_main_grad) \
+    X(puro_fp8_linear_backward)        \
+    X(puro_fp8_linear_dgrad_quantize)  \
+    X(puro_bf16_linear_fprop)          \
+    X(puro_bf16_linear_dgrad)          \
+    X(puro_bf16_linear_wgrad)
+struct Library {
+#define PURO_FIELD(name) decltype(&::name) name;
+    PURO_ENTRIES(PURO_FIELD)
+#undef PURO_FIELD
+};
+Library lib{};
+bool have_library = false;
+
 // `ok` is cleared when an argument is not of the ordinary kind: the call is left to Python.
 struct Args {
     PyObject *const *v;
@@ -146,7 +172,7 @@ PyObject *finish(const Args &a, F call) {
 
 #define PURO_NATIVE(name, nargs)                                                               \
     PyObject *name(PyObject *, PyObject *const *argv, Py_ssize_t n) {                          \
-        if (n != (nargs)) Py_RETURN_NONE;                                                      \
+        if (n != (nargs) || !have_library) Py_RETURN_NONE;                                     \
         Args a{argv};                                                                          \
         try {                                                                                  \
             return name##_call(a);                                                             \
@@ -166,7 +192,7 @@ PyObject *amax_call(Args &a) {
     int64_t r, c;
     a.shape(0, &r, &c);
     void *s = a.stream(2);
-    return finish(a, [&] { return puro_fp8_amax(x, r, c, bits, s); });
+    return finish(a, [&] { return lib.puro_fp8_amax(x, r, c, bits, s); });
 }
 PURO_NATIVE(amax, 3)
 
@@ -182,7 +208,7 @@ PyObject *quantize_call(Args &a) {
     void *sc = a.opt(6, sdt), *sct = a.opt(8, sdt);
     int32_t *st = a.status(9);
     void *s = a.stream(10);
-    return finish(a, [&] { return puro_fp8_quantize(x, r, c, fmt, scaling, role, bits, q, sc, qt, sct, st, s); });
+    return finish(a, [&] { return lib.puro_fp8_quantize(x, r, c, fmt, scaling, role, bits, q, sc, qt, sct, st, s); });
 }
 PURO_NATIVE(quantize, 11)
 
@@ -198,7 +224,7 @@ PyObject *quantize_rmsnorm_call(Args &a) {
     uint8_t *q = u8(a.opt(6, kU8)), *qt = u8(a.opt(8, kU8));
     int32_t *st = a.status(10);
     void *s = a.stream(11);
-    return finish(a, [&] { return puro_fp8_quantize_rmsnorm(h, r, c, gamma, eps, fmt, rstd, y, q, sc, qt, sct, st, s); });
+    return finish(a, [&] { return lib.puro_fp8_quantize_rmsnorm(h, r, c, gamma, eps, fmt, rstd, y, q, sc, qt, sct, st, s); });
 }
 PURO_NATIVE(quantize_rmsnorm, 12)
 
@@ -216,7 +242,7 @@ PyObject *quantize_swiglu_call(Args &a) {
     int32_t *st = a.status(8);
     void *s = a.stream(9);
     return finish(a, [&] {
-        return puro_fp8_quantize_swiglu(g->data_ptr(), u->data_ptr(), g->size(0), g->size(1), g->stride(0), fmt, y, q,
+        return lib.puro_fp8_quantize_swiglu(g->data_ptr(), u->data_ptr(), g->size(0), g->size(1), g->stride(0), fmt, y, q,
                                         sc, qt, sct, st, s);
     });
 }
@@ -229,7 +255,7 @@ PyObject *quantize_weights_call(Args &a) {
     int32_t *st = a.status(3);
     void *s = a.stream(4);
     return finish(a, [&] {
-        return puro_fp8_quantize_weights(reinterpret_cast<const puro_fp8_weight_t *>(table), count, fmt, st, s);
+        return lib.puro_fp8_quantize_weights(reinterpret_cast<const puro_fp8_weight_t *>(table), count, fmt, st, s);
     });
 }
 PURO_NATIVE(quantize_weights, 5)
@@ -247,14 +273,14 @@ PyObject *gemm(Args &a, Fn fn, at::ScalarType out_dtype) {
     void *s = a.stream(5);
     return finish(a, [&] { return fn(&x, &w, out, ws, bytes, st, s); });
 }
-PyObject *linear_fprop_call(Args &a) { return gemm(a, puro_fp8_linear_fprop, kBF16); }
-PyObject *linear_dgrad_call(Args &a) { return gemm(a, puro_fp8_linear_dgrad, kBF16); }
-PyObject *linear_wgrad_call(Args &a) { return gemm(a, puro_fp8_linear_wgrad, kBF16); }
+PyObject *linear_fprop_call(Args &a) { return gemm(a, lib.puro_fp8_linear_fprop, kBF16); }
+PyObject *linear_dgrad_call(Args &a) { return gemm(a, lib.puro_fp8_linear_dgrad, kBF16); }
+PyObject *linear_wgrad_call(Args &a) { return gemm(a, lib.puro_fp8_linear_wgrad, kBF16); }
 PyObject *linear_wgrad_main_grad_call(Args &a) {
     return gemm(a,
                 [](const puro_fp8_tensor_t *x, const puro_fp8_tensor_t *w, void *out, void *ws, size_t bytes, int32_t *st,
                    void *s) {
-                    return puro_fp8_linear_wgrad_main_grad(x, w, static_cast<float *>(out), ws, bytes, st, s);
+                    return lib.puro_fp8_linear_wgrad_main_grad(x, w, static_cast<float *>(out), ws, bytes, st, s);
                 },
                 kF32);
 }
@@ -276,7 +302,7 @@ PyObject *linear_backward_call(Args &a) {
     void *ws = a.scratch(6, &bytes);
     int32_t *st = a.status(7);
     void *s = a.stream(8);
-    return finish(a, [&] { return puro_fp8_linear_backward(&dy, &wt, dx, &dyt, &xt, dw, ws, bytes, st, s); });
+    return finish(a, [&] { return lib.puro_fp8_linear_backward(&dy, &wt, dx, &dyt, &xt, dw, ws, bytes, st, s); });
 }
 PURO_NATIVE(linear_backward, 9)
 
@@ -290,7 +316,7 @@ PyObject *linear_dgrad_quantize_call(Args &a) {
     uint8_t *q = u8(a.opt(4, kU8)), *qt = u8(a.opt(6, kU8));
     int32_t *st = a.status(8);
     void *s = a.stream(9);
-    return finish(a, [&] { return puro_fp8_linear_dgrad_quantize(&dy, &wt, fmt, dx, q, sc, qt, sct, st, s); });
+    return finish(a, [&] { return lib.puro_fp8_linear_dgrad_quantize(&dy, &wt, fmt, dx, q, sc, qt, sct, st, s); });
 }
 PURO_NATIVE(linear_dgrad_quantize, 10)
 
@@ -304,9 +330,9 @@ PyObject *bf16(Args &a, Fn fn) {
     void *s = a.stream(7);
     return finish(a, [&] { return fn(x, w, out, M, N, K, st, s); });
 }
-PyObject *bf16_fprop_call(Args &a) { return bf16(a, puro_bf16_linear_fprop); }
-PyObject *bf16_dgrad_call(Args &a) { return bf16(a, puro_bf16_linear_dgrad); }
-PyObject *bf16_wgrad_call(Args &a) { return bf16(a, puro_bf16_linear_wgrad); }
+PyObject *bf16_fprop_call(Args &a) { return bf16(a, lib.puro_bf16_linear_fprop); }
+PyObject *bf16_dgrad_call(Args &a) { return bf16(a, lib.puro_bf16_linear_dgrad); }
+PyObject *bf16_wgrad_call(Args &a) { return bf16(a, lib.puro_bf16_linear_wgrad); }
 PURO_NATIVE(bf16_fprop, 8)
 PURO_NATIVE(bf16_dgrad, 8)
 PURO_NATIVE(bf16_wgrad, 8)
@@ -323,8 +349,33 @@ PyObject *set_operand_type(PyObject *, PyObject *const *argv, Py_ssize_t n) {
     Py_RETURN_NONE;
 }
 
+// (name -> address of each entry point)
+PyObject *set_library(PyObject *, PyObject *const *argv, Py_ssize_t n) {
+    if (n != 1 || !PyDict_Check(argv[0])) {
+        PyErr_SetString(PyExc_TypeError, "set_library takes one dict");
+        return nullptr;
+    }
+    Library l{};
+#define PURO_TAKE(name)                                                                    \
+    {                                                                                      \
+        PyObject *o = PyDict_GetItemString(argv[0], #name);                                \
+        void *p = o ? PyLong_AsVoidPtr(o) : nullptr;                                       \
+        if (!p) {                                                                          \
+            if (!PyErr_Occurred()) PyErr_SetString(PyExc_ValueError, "no address of " #name); \
+            return nullptr;                                                                \
+        }                                                                                  \
+        l.name = reinterpret_cast<decltype(l.name)>(p);                                    \
+    }
+    PURO_ENTRIES(PURO_TAKE)
+#undef PURO_TAKE
+    lib = l;
+    have_library = true;
+    Py_RETURN_NONE;
+}
+
 #define PURO_METHOD(py, fn) {py, reinterpret_cast<PyCFunction>(reinterpret_cast<void *>(fn)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {PURO_METHOD("set_operand_type", set_operand_type),
+                         PURO_METHOD("set_library", set_library),
                          PURO_METHOD("puro_fp8_amax", amax),
                          PURO_METHOD("puro_fp8_quantize", quantize),
                          PURO_METHOD("puro_fp8_quantize_rmsnorm", quantize_rmsnorm),

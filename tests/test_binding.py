@@ -3,6 +3,10 @@ argument that is not of the ordinary kind to the Python code (which raises or
 handles it), and for ordinary arguments both give the same bytes and errors.
 """
 import ctypes
+import importlib
+import os
+import shutil
+import sys
 
 import numpy as np
 import pytest
@@ -78,6 +82,50 @@ def test_native_refuses_other_operand_classes():
     b = _buffers("cpu")
     o = Sub(b["xo"].data, b["xo"].scale)
     assert P._load_native().puro_fp8_linear_fprop(o, b["wo"], b["y"], None, None, None) is None
+
+
+@pytest.fixture
+def copy_of_the_package(tmp_path):
+    """The package a second time in this process, from other files."""
+    shutil.copytree(os.path.dirname(P.__file__), tmp_path / "puro_copy",
+                    ignore=shutil.ignore_patterns("_build", "__pycache__"))
+    sys.path.insert(0, str(tmp_path))
+    try:
+        yield importlib.import_module("puro_copy")
+    finally:
+        sys.path.remove(str(tmp_path))
+        for name in [n for n in sys.modules if n.split(".")[0] == "puro_copy"]:
+            del sys.modules[name]
+
+
+def test_a_copy_of_the_package_brings_no_second_binding_to_the_library(copy_of_the_package):
+    C = copy_of_the_package
+    P._load_native(), C._load_native()
+    address = lambda lib: ctypes.cast(lib.puro_fp8_amax, ctypes.c_void_p).value  # noqa: E731
+    assert address(P.load_library()) != address(C.load_library())
+    # linked by name, the copy's module would find the library loaded first
+    with pytest.raises(AttributeError):
+        ctypes.CDLL(C._build.NATIVE).puro_fp8_amax
+
+
+@pytest.mark.gpu
+def test_a_copy_of_the_package_calls_its_own_library(copy_of_the_package):
+    """The wait bound set through one copy (by ctypes) holds for that copy's hot calls alone."""
+    C = copy_of_the_package
+    x = W.normal_bf16((4096, 4096), 1.0, DEV, 60)
+    got = {}
+    for bounded in (P, C):
+        bounded.puro_set_wait_timeout_ns(0)
+        try:
+            for p in (P, C):
+                status = torch.zeros(1, dtype=torch.int32, device=DEV)
+                q = p.quantize(x, p.E4M3)
+                p.puro_fp8_quantize(x, p.E4M3, p.SCALE_BLOCK, p.ROLE_ACT, None, q.rowwise.data, q.rowwise.scale,
+                                    q.colwise.data, q.colwise.scale, status)
+                got[bounded, p] = p.puro_fp8_get_status(status)
+        finally:
+            bounded.puro_set_wait_timeout_ns(2_000_000_000)
+    assert got == {(b, p): P.PURO_ERR_TIMEOUT if b is p else P.PURO_OK for b in (P, C) for p in (P, C)}
 
 
 def _random(b):
