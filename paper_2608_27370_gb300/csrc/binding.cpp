@@ -159,7 +159,8 @@ struct Args {
     }
 };
 
-// Runs `call` without the GIL when every argument was ordinary.
+// Runs `call` without the GIL when every argument was ordinary.  It touches no
+// tensor and must not throw: every pointer and size is taken before.
 template <class F>
 PyObject *finish(const Args &a, F call) {
     if (!a.ok) Py_RETURN_NONE;
@@ -236,15 +237,14 @@ PyObject *quantize_swiglu_call(Args &a) {
         g->sizes() != u->sizes() || g->size(0) < 2 || g->stride(1) != 1 || u->stride(1) != 1 ||
         g->stride(0) != u->stride(0))
         Py_RETURN_NONE;
+    const void *gp = g->data_ptr(), *up = u->data_ptr();
+    const int64_t r = g->size(0), c = g->size(1), ld = g->stride(0);
     const int32_t fmt = a.i32(2);
     void *y = a.opt(3, kBF16), *sc = a.opt(5, kU8), *sct = a.opt(7, kU8);
     uint8_t *q = u8(a.opt(4, kU8)), *qt = u8(a.opt(6, kU8));
     int32_t *st = a.status(8);
     void *s = a.stream(9);
-    return finish(a, [&] {
-        return lib.puro_fp8_quantize_swiglu(g->data_ptr(), u->data_ptr(), g->size(0), g->size(1), g->stride(0), fmt, y, q,
-                                        sc, qt, sct, st, s);
-    });
+    return finish(a, [&] { return lib.puro_fp8_quantize_swiglu(gp, up, r, c, ld, fmt, y, q, sc, qt, sct, st, s); });
 }
 PURO_NATIVE(quantize_swiglu, 10)
 

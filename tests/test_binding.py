@@ -6,6 +6,7 @@ import ctypes
 import importlib
 import os
 import shutil
+import subprocess
 import sys
 
 import numpy as np
@@ -14,6 +15,7 @@ import torch
 
 import paper_2608_27370_gb300 as P
 from paper_2608_27370_gb300 import workloads as W
+import _native_harness as H
 
 DEV = "cuda"
 u8, i32, bf16, f32 = torch.uint8, torch.int32, torch.bfloat16, torch.float32
@@ -82,6 +84,19 @@ def test_native_refuses_other_operand_classes():
     b = _buffers("cpu")
     o = Sub(b["xo"].data, b["xo"].scale)
     assert P._load_native().puro_fp8_linear_fprop(o, b["wo"], b["y"], None, None, None) is None
+
+
+@pytest.fixture(scope="module")
+def harness(tmp_path_factory):
+    """Path of the native module built to run without a GPU."""
+    return H.build(tmp_path_factory.mktemp("harness"))
+
+
+def test_native_declines_tensors_whose_memory_cannot_be_accessed(harness):
+    """In a process of its own: a function that throws without the interpreter's lock ends it."""
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join(p for p in sys.path if p))
+    r = subprocess.run([sys.executable, H.__file__, harness], capture_output=True, text=True, env=env)
+    assert r.returncode == 0 and r.stdout.split("\n")[-2] == "declined all", (r.returncode, r.stdout, r.stderr)
 
 
 @pytest.fixture
