@@ -6,7 +6,8 @@ tensors it is handed are CUDA, contiguous and of the right dtype, and passes
 their device pointers, the sizes and the current CUDA stream to the library
 entry point of the same name.  The calls of a training step do this in native
 code (``csrc/binding.cpp``) for ordinary arguments; anything else it hands
-back, and the ctypes path below it checks the arguments one by one.  All
+back, and the ctypes path below it checks the arguments one by one (as every
+call does where that module was compiled for another torch).  All
 arithmetic runs in the library's CUDA kernels.  There is no fallback: if the
 library is missing, every call raises.
 
@@ -23,6 +24,7 @@ import ctypes
 import importlib.machinery
 import importlib.util
 import os
+import warnings
 from dataclasses import dataclass
 from typing import Optional
 
@@ -126,17 +128,31 @@ def load_library(path: Optional[str] = None):
 _native = None
 
 
+class _CtypesOnly:
+    """Stands in for the native module: hands every call back."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
 def _load_native():
-    """The native marshalling module, calling the library that load_library() returns."""
+    """The native marshalling module, calling the library that load_library() returns.  Without
+    one for this torch and interpreter every call takes its ctypes path."""
     global _native
     lib = load_library()
-    if not os.path.exists(_build.NATIVE):
-        raise RuntimeError(f"{_build.NATIVE} not found: build it with "
-                           "`python -c 'import __graft_entry__ as g; g.build()'`")
     name = __name__ + "._native"
     loader = importlib.machinery.ExtensionFileLoader(name, _build.NATIVE)
-    module = importlib.util.module_from_spec(importlib.util.spec_from_loader(name, loader))
-    loader.exec_module(module)
+    try:
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader(name, loader))
+        loader.exec_module(module)
+        made_for = getattr(module, "native_for", "another version")
+        if made_for != _build.native_for():
+            raise ImportError(f"it was compiled for {made_for}, this is {_build.native_for()}")
+    except ImportError as e:
+        warnings.warn(f"calls are marshalled by ctypes (9 us more each), {_build.NATIVE} cannot be used: {e}; rebuild "
+                      "with `python -c 'import __graft_entry__ as g; g.build()'`", stacklevel=3)
+        _native = _CtypesOnly()
+        return _native
     module.set_operand_type(FP8Operand)
     module.set_library({n: ctypes.cast(getattr(lib, n), ctypes.c_void_p).value for n in _SIGNATURES})
     _native = module

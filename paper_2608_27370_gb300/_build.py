@@ -12,6 +12,7 @@ import concurrent.futures as cf
 import os
 import shutil
 import subprocess
+import sys
 import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -22,6 +23,7 @@ BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libpuro_fp8.so")
 NATIVE = os.path.join(PKG, "_native.so")
 BINDING = os.path.join(CSRC, "binding.cpp")
+NATIVE_FOR = os.path.join(BUILD, "native_for.txt")  # what _native.so was compiled for
 SOURCES = ["api.cu", "quantize.cu", "gemm.cu", "noalloc.cu", "muonh.cu"]
 HEADERS = ["ptx.cuh", "internal.h", "quant_math.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -36,9 +38,20 @@ def _nvcc() -> str:
     raise RuntimeError("nvcc not found: the CUDA toolkit is required to build libpuro_fp8.so")
 
 
+def native_for() -> str:
+    """The torch and the interpreter that _native.so has to be compiled for: neither keeps
+    its binary interface from one version to the next."""
+    import torch
+
+    return f"torch {torch.__version__}, {sys.implementation.cache_tag}"
+
+
 def _stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(NATIVE):
+    if not all(os.path.exists(f) for f in (LIB, NATIVE, NATIVE_FOR)):
         return True
+    with open(NATIVE_FOR) as f:
+        if f.read() != native_for():
+            return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
     deps = [BINDING] + [os.path.join(CSRC, f) for f in SOURCES + HEADERS] + [os.path.join(INCLUDE, "puro_fp8.h"),
                                                                   os.path.abspath(__file__)]
@@ -70,7 +83,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         inc = os.path.join(os.path.dirname(torch.__file__), "include")
         obj = os.path.join(BUILD, "binding.o")
         cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-fvisibility=hidden", "-Wall",
-               "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI, "-isystem", inc, "-isystem",
+               f'-DPURO_NATIVE_FOR="{native_for()}"', "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI, "-isystem", inc, "-isystem",
                os.path.join(inc, "torch", "csrc", "api", "include"), "-isystem", sysconfig.get_paths()["include"],
                "-isystem", os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include"),
                "-I", INCLUDE, "-c", BINDING, "-o", obj]
@@ -101,6 +114,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if r.returncode != 0:
         raise RuntimeError(f"link of the binding failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, NATIVE)
+    with open(NATIVE_FOR, "w") as f:
+        f.write(native_for())
     return LIB
 
 

@@ -396,4 +396,12 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", "Native argument marshal
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__native() { return PyModule_Create(&module); }
+// (native_for: the torch and the interpreter it was compiled for)
+PyMODINIT_FUNC PyInit__native() {
+    PyObject *m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "native_for", PURO_NATIVE_FOR) < 0) {
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
+}

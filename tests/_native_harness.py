@@ -47,7 +47,7 @@ def build(folder) -> str:
             f.write(text)
     torch_dir = os.path.dirname(torch.__file__)
     so = os.path.join(folder, "_harness.so")
-    subprocess.run(["g++", "-O0", "-std=c++17", "-fPIC", "-shared", "-I", folder,
+    subprocess.run(["g++", "-O0", "-std=c++17", "-fPIC", "-shared", "-I", folder, '-DPURO_NATIVE_FOR="harness"',
                     "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
                     "-isystem", os.path.join(torch_dir, "include"), "-isystem",
                     os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),

@@ -21,13 +21,6 @@ DEV = "cuda"
 u8, i32, bf16, f32 = torch.uint8, torch.int32, torch.bfloat16, torch.float32
 
 
-class _General:
-    """Stands in for the native module: every call goes to the general path."""
-
-    def __getattr__(self, name):
-        return lambda *a: None
-
-
 def _buffers(dev, M=256, N=384, K=128):
     e = lambda dt, *s: torch.zeros(s, dtype=dt, device=dev)  # noqa: E731
     op = lambda r, c, role=P.ROLE_ACT: P.FP8Operand(e(u8, r, c), e(u8, *P.scale_vec_shape(r, c)), role=role)  # noqa: E731
@@ -97,6 +90,23 @@ def test_native_declines_tensors_whose_memory_cannot_be_accessed(harness):
     env = dict(os.environ, PYTHONPATH=os.pathsep.join(p for p in sys.path if p))
     r = subprocess.run([sys.executable, H.__file__, harness], capture_output=True, text=True, env=env)
     assert r.returncode == 0 and r.stdout.split("\n")[-2] == "declined all", (r.returncode, r.stdout, r.stderr)
+
+
+@pytest.mark.parametrize("kind", ["another torch", "missing", "not a module"])
+def test_without_a_usable_native_module_calls_go_through_ctypes(kind, monkeypatch, tmp_path):
+    monkeypatch.setattr(P, "_native", None)
+    if kind == "another torch":
+        monkeypatch.setattr(torch, "__version__", "2.0.0")
+        assert P._build._stale()  # and it is rebuilt
+    else:
+        monkeypatch.setattr(P._build, "NATIVE", str(tmp_path / "_native.so"))
+        if kind == "not a module":
+            (tmp_path / "_native.so").write_text("x")
+    with pytest.warns(UserWarning, match="marshalled by ctypes"):
+        with pytest.raises(ValueError, match="must be a CUDA tensor"):
+            P.puro_fp8_amax(torch.zeros((4, 4), dtype=bf16), torch.zeros(1, dtype=i32))
+    with pytest.raises(ValueError, match="must be a CUDA tensor"):  # and says so once
+        P.puro_bf16_linear_fprop(*(torch.zeros((4, 4), dtype=bf16) for _ in range(3)), 4, 4, 4)
 
 
 @pytest.fixture
@@ -171,7 +181,7 @@ def test_both_paths_give_the_same_bytes():
     got = []
     native = P._native
     try:
-        for route in (native, _General()):
+        for route in (native, P._CtypesOnly()):
             P._native = route
             b = _buffers(DEV)
             _random(b)
@@ -196,7 +206,7 @@ def test_errors_are_the_same(route):
     b = _buffers(DEV)
     q = (b["xo"].data, b["xo"].scale, b["xt"].data, b["xt"].scale)
     try:
-        P._native = native if route == "native" else _General()
+        P._native = native if route == "native" else P._CtypesOnly()
         with pytest.raises(ValueError, match="x has dtype"):
             P.puro_fp8_quantize(b["x"].float(), 0, 1, 0, None, *q)
         with pytest.raises(ValueError, match="x must be contiguous"):
