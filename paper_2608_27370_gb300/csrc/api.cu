@@ -230,7 +230,8 @@ BackwardPlan plan_backward(int64_t M, int64_t N, int64_t K, size_t ws) {
         if (sw == 1)
             b.grouped = true;
         else
-            b.grouped = b.wgrad_unsplit = grouped_backward_faster(M, N, K, sw);
+            b.grouped = b.wgrad_unsplit =
+                (g_tile_n.load() || !wgrad_keeps_split(M, N, K)) && grouped_backward_faster(M, N, K, sw);
     }
     auto launches_of = [](int sp, int64_t r, int64_t c, int64_t red) {
         return sp > 1 && cluster_split(r, c, red, sp) == 1 ? 2 : 1;

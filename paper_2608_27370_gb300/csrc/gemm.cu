@@ -1596,6 +1596,21 @@ bool grouped_backward_faster(int64_t M, int64_t N, int64_t K, int w_splits) {
     return grouped < separate;
 }
 
+// An unsplit Wgrad sums up to four times as many products in one FP32
+// accumulator as a split one.  Against 64 bits, before the rounding to BF16, on
+// (M, N, K) = (4096, 128, 2688) to (8320, 256, 1792): 1.9e-7 to 8.9e-7 unsplit,
+// 0.6e-7 to 2.5e-7 split; after it 2e-4 of the values instead of 1e-4 are not the
+// exact sum's rounding.  So a Dgrad of at most two k-blocks (N <= 256) gets no
+// grouped launch that would cost its Wgrad the split, though that is mostly
+// faster ((5376, 256, 2048) 10.5 against 17.2 us, (4224, 256, 384) 8.6 against
+// 9.7, (6528, 256, 128) 11.0 against 10.3).  Where 224 columns a tile would need
+// more rounds for that Dgrad than 256, and for larger N, Wgrads have joined the
+// Dgrad unsplit since there are grouped launches, and do.
+bool wgrad_keeps_split(int64_t M, int64_t N, int64_t K) {
+    auto rounds = [&](int64_t width) { return (pair_tiles(M, K, width) + kSplitRefPairs - 1) / kSplitRefPairs; };
+    return N <= 256 && rounds(224) <= rounds(256);
+}
+
 cudaError_t launch_gemm(const GemmArgs &g, const GemmMaps &m, cudaStream_t s) {
     switch (g.kind) {
         case kGemmBF16: return launch_width<kGemmBF16, kGemmOutBF16>(g, m, s);

@@ -206,6 +206,9 @@ int64_t splitk_rows_per_chunk(int64_t M);  // M rounded up to a whole 256-row pa
 // schedule, Wgrad unsplit) than as two launches with the Wgrad split into
 // w_splits chunks.  Host-only, shape-only.
 bool grouped_backward_faster(int64_t M, int64_t N, int64_t K, int w_splits);
+// Whether a Wgrad that would split its reduction does so also where a grouped
+// launch is faster, for its sum's sake.  Host-only, shape-only.
+bool wgrad_keeps_split(int64_t M, int64_t N, int64_t K);
 // Tile width (256, 192 or 128) of an unsplit GEMM with K reduction bytes, and of
 // a linear's Dgrad and Wgrad in one launch.  Host-only, shape-only.
 int choose_tile_n(int64_t M, int64_t N, int64_t K);

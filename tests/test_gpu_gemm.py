@@ -282,6 +282,24 @@ def test_grouped_backward_equals_separate_calls(M, N, K):
     assert P.puro_fp8_get_status(status) == 0
 
 
+@pytest.mark.parametrize("M,N,K", [(5376, 256, 2048), (6528, 256, 128), (5632, 128, 5248)])
+def test_backward_keeps_the_split_of_a_wgrad_behind_a_short_dgrad(M, N, K):
+    """dW has the bits of the Wgrad alone, which splits its reduction (on chip or through memory)."""
+    x, w, dy = _inputs(M, N, K, 8500 + M, t3=True)
+    xq = P.quantize(x, P.E4M3, P.SCALE_BLOCK, P.ROLE_ACT)
+    wq = P.quantize(w, P.E4M3, P.SCALE_BLOCK, P.ROLE_WEIGHT)
+    dyq = P.quantize(dy, P.E4M3, P.SCALE_BLOCK, P.ROLE_ACT)
+    ws = torch.full((P.puro_fp8_workspace_size(N, K, M),), 0xFF, dtype=torch.uint8, device=DEV)
+    dx = torch.empty((M, K), dtype=torch.bfloat16, device=DEV)
+    dw, dw1, dw2 = (torch.empty((N, K), dtype=torch.bfloat16, device=DEV) for _ in range(3))
+    P.puro_fp8_linear_backward(dyq.rowwise, wq.colwise, dx, dyq.colwise, xq.colwise, dw, ws)
+    P.puro_fp8_linear_wgrad(dyq.colwise, xq.colwise, dw1, ws)
+    P.puro_fp8_linear_wgrad(dyq.colwise, xq.colwise, dw2)
+    torch.cuda.synchronize()
+    assert torch.equal(dw.view(torch.int16), dw1.view(torch.int16))
+    assert not torch.equal(dw.view(torch.int16), dw2.view(torch.int16)), "the unsplit sum can be told apart"
+
+
 # Tile widths below 256 (chosen where they take fewer idle SM pairs): 128 at
 # few tiles, 192 at nine rows of tiles; the last tile of a row is cut, and the
 # 192-wide tiles start at row 64 of every other 128-row scale chunk.

@@ -213,6 +213,20 @@ def test_backward_plan_groups_every_c5_and_c6_linear(lib):
     assert lib.puro_fp8_linear_backward_launches(512, 32768, 256, 0) == 1  # no workspace: both unsplit, grouped
 
 
+# (M, N, K) and launches: a Wgrad of these that splits its reduction keeps it
+# behind a Dgrad of at most two k-blocks (split in a cluster: one launch, through
+# memory: two), but where that Dgrad has fewer rounds at 256 columns a tile than
+# at 224, and for three k-blocks.
+@pytest.mark.parametrize("M,N,K,launches", [(4224, 256, 384, 2), (5376, 256, 2048, 2), (6528, 256, 128, 2),
+                                            (5632, 128, 5248, 3), (7936, 256, 3712, 3), (4608, 128, 1024, 1),
+                                            (4736, 256, 1024, 1), (5504, 384, 128, 1), (5888, 384, 384, 1)])
+def test_backward_plan_keeps_the_split_of_a_wgrad_behind_a_short_dgrad(lib, M, N, K, launches):
+    ws = lib.puro_fp8_workspace_size(N, K, M)
+    assert ws > 0, "the Wgrad alone splits"
+    assert lib.puro_fp8_linear_backward_launches(M, N, K, ws) == launches
+    assert lib.puro_fp8_linear_backward_launches(M, N, K, ws - 1) == 1  # no room to split: grouped
+
+
 def test_bf16_gemm_validation(lib):
     assert lib.puro_bf16_linear_fprop(A, A, A, 12, 16, 16, None, None) == BAD   # M % 8
     assert lib.puro_bf16_linear_fprop(A, A + 2, A, 16, 16, 16, None, None) == BAD
