@@ -54,35 +54,80 @@ def _native_args(b, M=256, N=384, K=128):
     }
 
 
-@pytest.mark.parametrize("name", sorted(_native_args(_buffers("cpu"))))
-def test_native_leaves_unusual_arguments_alone(name):
-    native = P._load_native()
-    fn, args = getattr(native, name), list(_native_args(_buffers("cpu"))[name])
-    assert fn() is None and fn(*args, None) is None  # another number of arguments
-    if name != "puro_fp8_quantize_weights":
-        assert fn(*args) is None  # host tensors
-    odd = [object(), "x", 1.5, True, 2 ** 70, np.zeros(4), torch.zeros(0), torch.zeros(4, device="meta"),
-           torch.zeros(4, 4).t(), torch.nested.nested_tensor([torch.zeros(2)])]
-    for k in range(len(args)):
-        for o in odd:
-            if name == "puro_fp8_quantize_weights" and k == 0:
-                continue  # an address is taken as it is
-            assert fn(*args[:k], o, *args[k + 1:]) is None, (k, type(o))
-
-
-def test_native_refuses_other_operand_classes():
-    class Sub(P.FP8Operand):
-        pass
-
-    b = _buffers("cpu")
-    o = Sub(b["xo"].data, b["xo"].scale)
-    assert P._load_native().puro_fp8_linear_fprop(o, b["wo"], b["y"], None, None, None) is None
-
-
 @pytest.fixture(scope="module")
 def harness(tmp_path_factory):
     """Path of the native module built to run without a GPU."""
     return H.build(tmp_path_factory.mktemp("harness"))
+
+
+def _odd_arguments(m):
+    """What an argument may be instead, ordinary for some of them; m shows tensors as CUDA ones."""
+    whole = torch.zeros(64, 64)
+    yield from (None, object(), "x", 1.5, float("inf"), 3, True, 2 ** 31, 2 ** 70, np.zeros(4), whole, torch.zeros(0),
+                torch.zeros(4, device="meta"), torch.nested.nested_tensor([torch.zeros(2)]))
+    for dt in (bf16, f32, u8, i32, torch.uint32, torch.float64, torch.int64):
+        yield m.as_cuda(torch.zeros((2, 3), dtype=dt))
+        yield m.as_cuda(torch.zeros((256, 128), dtype=dt))
+    yield from (m.as_cuda(t) for t in (whole.t(), whole[:, :8], torch.zeros(0), torch.zeros(2, 3, 4, dtype=bf16),
+                                       torch.zeros(6, dtype=bf16), torch.zeros(128, 512, dtype=bf16).t(),
+                                       torch.zeros(256, 512, dtype=bf16)[:, :128]))
+    yield torch.nn.Parameter(m.as_cuda(torch.zeros((256, 128), dtype=bf16)))
+    codes, scale = m.as_cuda(torch.zeros((8, 16), dtype=u8)), m.as_cuda(torch.zeros(4))
+    yield from (P.FP8Operand(codes, scale, 1, 0, 1), P.FP8Operand(codes, m.as_cuda(whole.t())),
+                P.FP8Operand(m.as_cuda(torch.zeros(8, dtype=u8)), scale), P.FP8Operand(codes.view(torch.int8), scale),
+                P.FP8Operand(codes, torch.zeros(4)), P.FP8Operand(codes, None), P.FP8Operand(codes, scale, True),
+                P.FP8Operand(codes, scale, 2 ** 40))
+    yield type("Other", (P.FP8Operand,), {})(codes, scale)
+
+
+@pytest.mark.parametrize("name", sorted(_native_args(_buffers("cpu"))))
+def test_native_calls_the_library_as_ctypes_does(name, harness, monkeypatch):
+    """Ordinary arguments are accepted; whatever is accepted reaches the library with the arguments
+    of the general path; nothing else reaches it.  Every argument in turn is replaced."""
+    lib = H.Recorder()
+    m = H.load(harness, lib.addresses)
+    monkeypatch.setattr(P, "_lib", lib)
+    monkeypatch.setattr(P, "_native", P._CtypesOnly())
+    monkeypatch.setattr(P, "_stream", lambda stream: H.STREAM if stream is None else int(stream))
+    fn, table = getattr(m, name), (P.puro_fp8_weight_t * 1)()
+    table.count = 1
+    ordinary = [H.shown_as_cuda(m, a) for a in _native_args(_buffers("cpu"))[name]]
+    if name == "puro_fp8_quantize_weights":
+        ordinary[0] = ctypes.addressof(table)
+
+    def same(args):
+        """Whether the native function accepted; if so, compared."""
+        lib.calls.clear()
+        got = fn(*args)
+        if got is None:
+            assert not lib.calls
+            return False
+        assert got == lib.STATUS
+        if name == "puro_fp8_quantize_weights":
+            args = [table, *args[2:]] if args[:2] == ordinary[:2] else None
+        if args is not None:
+            with pytest.raises(P.PuroError):
+                getattr(P, name)(*args)
+            native, general = lib.calls
+            assert native == general
+        return True
+
+    assert same(ordinary)
+    assert fn() is None and fn(*ordinary, None) is None  # another number of arguments
+    for k, a in enumerate(ordinary):
+        for odd in _odd_arguments(m):
+            if name == "puro_fp8_quantize_weights" and k < 2:
+                continue  # made by the binding
+            accepted = same([*ordinary[:k], odd, *ordinary[k + 1:]])
+            if type(odd) in (object, str, bool, np.ndarray) or (torch.is_tensor(odd) and not odd.is_cuda):
+                assert not accepted
+
+
+def test_native_refuses_an_incomplete_library(harness):
+    lib = H.Recorder()
+    m = H.load(harness, lib.addresses)
+    with pytest.raises(ValueError, match="no address of puro_bf16_linear_wgrad"):
+        m.set_library({k: v for k, v in lib.addresses.items() if k != "puro_bf16_linear_wgrad"})
 
 
 def test_native_declines_tensors_whose_memory_cannot_be_accessed(harness):
@@ -185,6 +230,10 @@ def test_both_paths_give_the_same_bytes():
             P._native = route
             b = _buffers(DEV)
             _random(b)
+            if route is native:  # they are taken, not handed back
+                for name, args in _native_args(b).items():
+                    assert getattr(native, name)(*args) == P.PURO_OK, name
+                b["main"].zero_()
             for name, call in _calls(b):
                 call()
             torch.cuda.synchronize()

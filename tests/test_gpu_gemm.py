@@ -300,6 +300,76 @@ def test_backward_keeps_the_split_of_a_wgrad_behind_a_short_dgrad(M, N, K):
     assert not torch.equal(dw.view(torch.int16), dw2.view(torch.int16)), "the unsplit sum can be told apart"
 
 
+def _assert_tile_width(width, call):
+    """The GEMM kernels that call launches run at this tile width (from the kernel's name, where the
+    machine lets a profiler see it)."""
+    from torch.profiler import ProfilerActivity, profile
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    names = [e.name() for e in prof.profiler.kineto_results.events() if "gemm_tn_kernel" in e.name()]
+    widths = {int(n.split("gemm_tn_kernel<")[1].split(">")[0].split(",")[2].split(")")[-1]) for n in names}
+    assert widths <= {width}, (names, width)
+
+
+# Narrow tiles in a grouped launch, more units than pairs: the Dgrad's or the
+# Wgrad's units the long ones, fewer of them than pairs, so that the other pairs
+# take short ones first.
+@pytest.mark.parametrize("M,N,K,width", [(256, 2048, 1536, 128), (1152, 3072, 640, 128), (4480, 384, 512, 128),
+                                         (256, 768, 3840, 192), (640, 2304, 1792, 192), (2048, 384, 2816, 192)])
+def test_grouped_backward_narrow_tiles(M, N, K, width):
+    x, w, dy = _inputs(M, N, K, 8600 + M + N + K, t3=True)
+    xq = P.quantize(x, P.E4M3, P.SCALE_BLOCK, P.ROLE_ACT)
+    wq = P.quantize(w, P.E4M3, P.SCALE_BLOCK, P.ROLE_WEIGHT)
+    dyq = P.quantize(dy, P.E4M3, P.SCALE_BLOCK, P.ROLE_ACT)
+    dx, dw = (torch.full(s, float("nan"), dtype=torch.bfloat16, device=DEV) for s in ((M, K), (N, K)))
+    dx1, dw1 = torch.empty_like(dx), torch.empty_like(dw)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    call = lambda: P.puro_fp8_linear_backward(dyq.rowwise, wq.colwise, dx, dyq.colwise, xq.colwise, dw,  # noqa: E731
+                                              dev_status=status)
+    assert P.puro_fp8_linear_backward_launches(M, N, K, 0) == 1
+    call()
+    P.puro_fp8_linear_dgrad(dyq.rowwise, wq.colwise, dx1)
+    P.puro_fp8_linear_wgrad(dyq.colwise, xq.colwise, dw1)
+    torch.cuda.synchronize()
+    assert P.puro_fp8_get_status(status) == 0
+    assert torch.equal(dx.view(torch.int16), dx1.view(torch.int16)), "dX differs from the separate Dgrad"
+    assert torch.equal(dw.view(torch.int16), dw1.view(torch.int16)), "dW differs from the separate Wgrad"
+    ref = oracle_linear(x, w, dy, P.SCALE_BLOCK)
+    assert_close(dx, ref["dx"], "grouped dgrad")
+    assert_close(dw, ref["dw"], "grouped wgrad")
+    _assert_tile_width(width, call)
+
+
+# More narrow tiles than SM pairs: 39 x 3 of 128 columns, 16 x 8 of 192 columns.
+@pytest.mark.parametrize("M,N,K,width", [(9984, 384, 384, 128), (4096, 1536, 640, 192)])
+@pytest.mark.parametrize("kind", ["block", "tensor", "bf16", "block main-grad", "tensor main-grad"])
+def test_gemm_narrow_tiles_several_a_pair(M, N, K, width, kind):
+    x, w, _ = _inputs(M, N, K, 8650 + M, t3=True)
+    main_grad, start = kind.endswith("main-grad"), 0
+    out = W.normal_f32((M, N), 1.0, DEV, 8660) if main_grad else torch.empty((M, N), dtype=torch.bfloat16, device=DEV)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    if kind == "bf16":
+        call = lambda: P.puro_bf16_linear_fprop(x, w, out, M, N, K, status)  # noqa: E731
+        A, B = (O.bf16_to_double(bits(t)) for t in (x, w))
+    else:
+        scaling = P.SCALE_BLOCK if kind.startswith("block") else P.SCALE_TENSOR
+        xq, wq = (P.quantize(t, P.E4M3, scaling, P.ROLE_ACT) for t in (x, w))
+        gemm = P.puro_fp8_linear_wgrad_main_grad if main_grad else P.puro_fp8_linear_fprop
+        call = lambda: gemm(xq.rowwise, wq.rowwise, out, None, status)  # noqa: E731
+        if scaling == P.SCALE_BLOCK:
+            A, B = (O.dequant_rows_1x128(*par_quantize_rows_1x128(bits(t), P.E4M3), P.E4M3) for t in (x, w))
+        else:
+            A, B = (O.dequant_tensor(*O.quantize_tensor(bits(t), P.E4M3)[1:], P.E4M3) for t in (x, w))
+    if main_grad:
+        start = out.double()
+    call()
+    torch.cuda.synchronize()
+    assert P.puro_fp8_get_status(status) == 0
+    check_gemm_every_tile(out.double() - start if main_grad else out, A, B, np.random.default_rng(8670 + M), kind)
+    _assert_tile_width(width, call)
+
+
 # Tile widths below 256 (chosen where they take fewer idle SM pairs): 128 at
 # few tiles, 192 at nine rows of tiles; the last tile of a row is cut, and the
 # 192-wide tiles start at row 64 of every other 128-row scale chunk.

@@ -109,3 +109,29 @@ def test_fused_rmsnorm_with_an_unaligned_rstd(write_y):
         got.append([rstd, y.view(torch.int16), q.rowwise.data, q.rowwise.scale, q.colwise.data, q.colwise.scale])
     for other in got[1:]:
         assert all(torch.equal(a, b) for a, b in zip(got[0], other))
+
+
+def test_fused_rmsnorm_right_behind_a_gemm_that_writes_h():
+    """The quantiser loads its first tile of h ahead of its wait, which holds because the rstd pass
+    before it has waited for the kernel that writes h: here a GEMM, over other values each time."""
+    rows, cols, k = 1024, 2048, 512
+    gamma = W.normal_f32((cols,), 0.1, DEV, 962).add_(1.0).to(torch.bfloat16)
+    a = [W.normal_bf16((rows, k), 1.0, DEV, 970 + i) for i in range(4)]
+    b = W.normal_bf16((cols, k), 0.05, DEV, 980)
+    h = torch.zeros((rows, cols), dtype=torch.bfloat16, device=DEV)
+
+    def outputs(sync):
+        got = []
+        for x in a:
+            rstd, q = torch.empty(rows, dtype=torch.float32, device=DEV), _empty_q(rows, cols)
+            P.puro_bf16_linear_fprop(x, b, h, rows, cols, k)
+            if sync:
+                torch.cuda.synchronize()
+            P.puro_fp8_quantize_rmsnorm(h, gamma, 1e-6, P.E4M3, rstd, None, q.rowwise.data, q.rowwise.scale,
+                                        q.colwise.data, q.colwise.scale)
+            got += [rstd, q.rowwise.data, q.rowwise.scale, q.colwise.data, q.colwise.scale]
+        torch.cuda.synchronize()
+        return got
+
+    for _ in range(5):
+        assert all(torch.equal(s, t) for s, t in zip(outputs(False), outputs(True)))
