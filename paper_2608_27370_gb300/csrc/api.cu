@@ -144,7 +144,7 @@ puro_status_t prepare_fp8_gemm(const puro_fp8_tensor_t *a, const puro_fp8_tensor
     if (!make_map(&m.a, CU_TENSOR_MAP_DATA_TYPE_UINT8, a->data, K, M, K, kGemmBKBytes, kGemmBM,
                   CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map(&m.b, CU_TENSOR_MAP_DATA_TYPE_UINT8, b->data, K, N, K, kGemmBKBytes,
-                  static_cast<uint32_t>(block && tile_n == 256 ? 64 : tile_n / 2), CU_TENSOR_MAP_SWIZZLE_128B) ||
+                  static_cast<uint32_t>(tile_n / 2), CU_TENSOR_MAP_SWIZZLE_128B) ||
         !(accumulate_f32
               ? make_map(&m.d, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, d, N, M, N * 4, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B)
               : make_map(&m.d, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, d, N, M, N * 2, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B)))

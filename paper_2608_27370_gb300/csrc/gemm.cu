@@ -38,9 +38,15 @@
 //                     buffers do not fit: tiles alternate between columns
 //                     [0, 256) and [128, 384), sharing [128, 256).  The
 //                     epilogue reads the shared half first and releases the
-//                     accumulator as soon as that half is in registers; the
-//                     tile's last MMAs are issued for that half first, so that
-//                     its drain overlaps the other half's.
+//                     accumulator as soon as that half is in registers, so
+//                     the next tile's MMAs wait for half a drain.  (The last
+//                     k-blocks as two 128-wide halves, the shared one first,
+//                     would hide that: [8192, 2048] x 2048 23.4 -> 22.7 us, a
+//                     whole linear of that size 112.2 -> 111.4, one of 640
+//                     tokens 28.7 -> 29.1.  But PTX runs two MMAs on one
+//                     accumulator in the order of issue only if their shapes
+//                     are equal, and with a wait between the shapes it takes
+//                     24.4.)
 //   block, narrower   two independent buffers at columns 0 and 256 (scale
 //                     vectors at 480): the next tile never waits for a drain.
 //                     The host picks a narrower form where the 256-wide tiles
@@ -68,7 +74,6 @@ constexpr int kThreads = 256;
 constexpr int kTmemCols = 512;
 constexpr int kSfColsPerSet = 12;  // 4 for A (128 rows) + 8 for B (up to 256 rows)
 constexpr int kSfSets = 2;         // double-buffered across groups of four k-blocks
-constexpr int kTailBlocks = 3;     // k-blocks of a shifted tile issued as halves
 constexpr uint32_t kPrefetchNs = 100;  // pause between the k-blocks of B a waiting CTA prefetches
 constexpr int64_t kPrefetchBytes = 8 << 20;  // a smaller B is not worth the prologue's time (0.1 us)
 constexpr uint32_t kAllocBarrier = 7, kLeaveBarrier = 8;  // named barriers (the quantising epilogue uses 1..6)
@@ -131,10 +136,7 @@ struct GemmSmem {
     alignas(128) uint8_t sf_b[kSfbByHelper ? kSfbSlots : kStages][512 * kSfbChunks];
     uint64_t full[kStages];   // even CTA: both CTAs' copies of a stage landed
     uint64_t empty[kStages];  // both CTAs: the pair MMAs reading a stage are done
-    // both CTAs: accumulator complete.  Shifted: [0] the shared half, [1 + tile
-    // parity] the other one (its wait may come after the next tile's MMAs are
-    // done, so consecutive tiles use two barriers)
-    uint64_t tfull[3];
+    uint64_t tfull[2];        // both CTAs: accumulator complete
     uint64_t tempty[2];       // even CTA: both CTAs' epilogues released the accumulator
     uint64_t sfb_full[kSfbSlots];   // even CTA (BN = 224): both CTAs' B scale images built
     uint64_t sfb_empty[kSfbSlots];  // both CTAs (BN = 224): the copies reading an image are done
@@ -567,10 +569,6 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
     // 256-wide form 0.5%).
     constexpr bool kEarlyLeave = BN < 256 && !OUT_Q;
     constexpr bool kShifted = kMX && BN == 256;         // shared-half accumulators
-    // Shifted accumulators: the tile's last k-blocks are issued as two 128-wide
-    // halves, the shared one first (see the MMA issuer).
-    constexpr int kTail = kShifted && !OUT_Q ? kTailBlocks : 0;
-    constexpr int kBoxRows = kTail ? 64 : kBNHalf;      // rows of a B copy
     constexpr int kAccBufs = kShifted ? 1 : 2;          // hand-off barrier pairs (tfull / tempty)
     constexpr int kAccShift = kShifted ? 128 : 256;     // column offset between consecutive tiles' accumulators
     constexpr int kSfBase = kShifted ? 384 : 480;       // first scale-vector column (MX)
@@ -613,8 +611,10 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
             mbar_init(&sm.full[s], 1);
             mbar_init(&sm.empty[s], 1);
         }
-        for (int b = 0; b < 3; ++b) mbar_init(&sm.tfull[b], 1);
-        for (int b = 0; b < 2; ++b) mbar_init(&sm.tempty[b], OUT_Q ? 32 : 8);  // the epilogue warps of both CTAs
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&sm.tfull[b], 1);
+            mbar_init(&sm.tempty[b], OUT_Q ? 32 : 8);  // the epilogue warps of both CTAs
+        }
         for (int s = 0; s < kSfbSlots; ++s) {
             mbar_init(&sm.sfb_full[s], 2);  // the helper warp of each CTA
             mbar_init(&sm.sfb_empty[s], 1);
@@ -726,18 +726,7 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
 #pragma unroll
                 for (int at = 0; at < kAtoms; ++at) {
                     tma_load_2d_pair_e(e, sm.a[stage][at], ma, full_bar, kb * kBK + at * kAtomK, a_row);
-                    if constexpr (kTail > 0) {
-                        // 64 rows at a time: the CTA's half of the tile's rows, but in the
-                        // last k-blocks its half of each 128-row half
-                        const bool tail = kb >= wu.kb1 - kTail;
-                        const int row0 = tail ? wu.n0 + kBoxRows * static_cast<int>(rank) : b_row;
-                        const int row1 = row0 + (tail ? 2 : 1) * kBoxRows;
-                        tma_load_2d_pair_e(e, sm.b[stage][at], mb, full_bar, kb * kBK + at * kAtomK, row0);
-                        tma_load_2d_pair_e(e, sm.b[stage][at] + kBoxRows * kAtomBytes, mb, full_bar,
-                                         kb * kBK + at * kAtomK, row1);
-                    } else {
-                        tma_load_2d_pair_e(e, sm.b[stage][at], mb, full_bar, kb * kBK + at * kAtomK, b_row);
-                    }
+                    tma_load_2d_pair_e(e, sm.b[stage][at], mb, full_bar, kb * kBK + at * kAtomK, b_row);
                 }
                 if (sf_load) {
                     // chunks beyond the operand's rows read as zero (their rows are zero too)
@@ -785,30 +774,28 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
         // 2-10%: [32768, 2048] x 1536 71.9 -> 68.4 us, grouped backward of
         // (640, 1152, 2560) 11.1 -> 10.0).
         const uint32_t e = elect_one();
-        auto set_of = [&](int kb) { return static_cast<uint32_t>(kSfBase + ((kb / kStagesPerGroup) & 1) * kSfColsPerSet); };
-        auto copy_scales = [&](int kb, uint32_t stage, uint32_t slot) {  // a new group of four k-blocks: its scale vectors
-            const uint32_t sfa_col = set_of(kb), sfb_col = sfa_col + 4;
-            const uint8_t *sfb_src = kHelper ? sm.sf_b[slot] : sm.sf_b[stage];
-            tmem_cp_pair_32x128b_warpx4_e(e, tmem + sfa_col, smem_desc_plain_16B_rows(smem_u32(sm.sf_a[stage])));
-            tmem_cp_pair_32x128b_warpx4_e(e, tmem + sfb_col, smem_desc_plain_16B_rows(smem_u32(sfb_src)));
-            if constexpr (Smem::kSfbChunks == 2)
-                tmem_cp_pair_32x128b_warpx4_e(e, tmem + sfb_col + 4, smem_desc_plain_16B_rows(smem_u32(sfb_src + 512)));
-        };
-        // The MMAs of a stage on the columns of B that start at smem offset
-        // b_off (64 rows of each CTA per half), into d_tmem; the scale columns
-        // of B start sfb_shift into the set.
-        auto issue_mmas = [&](const WorkUnit &wu, int kb, uint32_t stage, uint32_t d_tmem, uint32_t idesc0, uint32_t b_off,
-                              uint32_t sfb_shift) {
-            const uint32_t sfa_col = set_of(kb), sfb_col = sfa_col + 4 + sfb_shift;
+        auto issue_stage = [&](const WorkUnit &wu, int kb, uint32_t stage, bool group_start, uint32_t slot,
+                               uint32_t d_tmem) {
+            const uint32_t sfa_col = static_cast<uint32_t>(kSfBase + ((kb / kStagesPerGroup) & 1) * kSfColsPerSet);
+            const uint32_t sfb_col = sfa_col + 4;
+            // a 192-wide tile starts at row 0 or 64 of its first 128-row scale chunk: 32 rows per column
+            const uint32_t sfb_shift = BN == 192 ? static_cast<uint32_t>(wu.n0 % 128) / 32u : 0u;
+            if (group_start) {  // a new group of four k-blocks: its scale vectors
+                const uint8_t *sfb_src = kHelper ? sm.sf_b[slot] : sm.sf_b[stage];
+                tmem_cp_pair_32x128b_warpx4_e(e, tmem + sfa_col, smem_desc_plain_16B_rows(smem_u32(sm.sf_a[stage])));
+                tmem_cp_pair_32x128b_warpx4_e(e, tmem + sfb_col, smem_desc_plain_16B_rows(smem_u32(sfb_src)));
+                if constexpr (Smem::kSfbChunks == 2)
+                    tmem_cp_pair_32x128b_warpx4_e(e, tmem + sfb_col + 4, smem_desc_plain_16B_rows(smem_u32(sfb_src + 512)));
+            }
 #pragma unroll
             for (int at = 0; at < kAtoms; ++at) {
-                uint32_t idesc = idesc0;
+                uint32_t idesc = wu.problem ? p.idesc1 : p.idesc;
                 if constexpr (kMX) {
                     const uint32_t sf_id = static_cast<uint32_t>((kb * kAtoms + at) & 3);  // k-block in its group
                     idesc |= (sf_id << 29) | (sf_id << 4);
                 }
                 const uint32_t a_addr = smem_u32(sm.a[stage][at]);
-                const uint32_t b_addr = smem_u32(sm.b[stage][at]) + b_off;
+                const uint32_t b_addr = smem_u32(sm.b[stage][at]);
 #pragma unroll
                 for (int k = 0; k < kKSteps; ++k) {
                     const uint64_t ad = smem_desc_k_sw128(a_addr + 32 * k);
@@ -819,9 +806,12 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
                     else if constexpr (KIND == kGemmFP8Tensor)
                         mma_pair_f8_e(e, d_tmem, ad, bd, idesc, acc);
                     else
-                        mma_pair_mxf8_e(e, d_tmem, ad, bd, idesc, tmem + sfa_col, tmem + sfb_col, acc);
+                        mma_pair_mxf8_e(e, d_tmem, ad, bd, idesc, tmem + sfa_col, tmem + sfb_col + sfb_shift, acc);
                 }
             }
+            tc_commit_pair_multicast_e(e, &sm.empty[stage], both);  // stage reusable in both CTAs
+            // the scale image is free once its copies (issued above) are done
+            if (kHelper && group_start) tc_commit_pair_multicast_e(e, &sm.sfb_empty[slot], both);
         };
         uint32_t stage = 0, phase = 0;
         uint32_t gseq = 0;  // groups of four k-blocks started (BN = 224: slot of the scale ring)
@@ -834,80 +824,26 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
             const uint32_t acc_phase = static_cast<uint32_t>(local / kAccBufs) & 1u;
             aborted = !wait_unless_aborted(sm, &sm.tempty[buf], acc_phase ^ 1u, p.wait_ns);
             const uint32_t d_tmem = tmem + static_cast<uint32_t>((local & 1) * kAccShift);
-            const uint32_t idesc = wu.problem ? p.idesc1 : p.idesc;
-            // a 192-wide tile starts at row 0 or 64 of its first 128-row scale chunk: 32 rows per column
-            const uint32_t sfb_shift = BN == 192 ? static_cast<uint32_t>(wu.n0 % 128) / 32u : 0u;
-            const int kt = kTail > 0 ? max(wu.kb0, wu.kb1 - kTail) : wu.kb1;
-            // the operands of stage kb, and its group's scales, are there
-            auto stage_ready = [&](int kb) {
+            for (int kb = wu.kb0; kb < wu.kb1 && !aborted; ++kb) {
                 const bool group_start = kMX && ((kb % kStagesPerGroup) == 0 || (S > 1 && kb == wu.kb0));
                 const uint32_t slot = gseq % kSfbSlots;
-                if (!wait_unless_aborted(sm, &sm.full[stage], phase, p.wait_ns)) return false;
-                if (kHelper && group_start &&
-                    !wait_unless_aborted(sm, &sm.sfb_full[slot], (gseq / kSfbSlots) & 1u, p.wait_ns))
-                    return false;
+                aborted = !wait_unless_aborted(sm, &sm.full[stage], phase, p.wait_ns) ||
+                          (kHelper && group_start &&
+                           !wait_unless_aborted(sm, &sm.sfb_full[slot], (gseq / kSfbSlots) & 1u, p.wait_ns));
+                if (aborted) break;
                 tc_fence_after_sync();
-                if (group_start) copy_scales(kb, stage, slot);
-                return true;
-            };
-            auto next_stage = [&] {
+                issue_stage(wu, kb, stage, group_start, slot, d_tmem);
+                if (group_start) ++gseq;
                 if (++stage == kStages) {
                     stage = 0;
                     phase ^= 1u;
-                }
-            };
-            for (int kb = wu.kb0; kb < kt && !aborted; ++kb) {
-                if (!stage_ready(kb)) {
-                    aborted = true;
-                    break;
-                }
-                issue_mmas(wu, kb, stage, d_tmem, idesc, 0, sfb_shift);
-                tc_commit_pair_multicast_e(e, &sm.empty[stage], both);  // stage reusable in both CTAs
-                if (kHelper && (kb % kStagesPerGroup) == 0) {
-                    // the scale image is free once its copies (issued above) are done
-                    tc_commit_pair_multicast_e(e, &sm.sfb_empty[gseq % kSfbSlots], both);
-                    ++gseq;
-                }
-                next_stage();
-            }
-            if constexpr (kTail > 0) {
-                // The last k-blocks, first for the half of the columns whose
-                // tensor memory the next tile shares, then for the other half:
-                // the epilogue drains the shared half while the other one's
-                // MMAs run.  Their rows of B are laid out by halves (see the
-                // producer), so that a 128-wide pair MMA covers 128 consecutive
-                // columns.  Three k-blocks (768 cycles of the tensor pipe) cover
-                // most of the drain's 900; with two or four the gain is no
-                // larger.  [8192, 2048] x 2048 24.8 -> 23.7 us, [32768, 1536] x
-                // 1536 54.9 -> 52.9, grouped backward of (4096, 2048, 2048) 24.9
-                // -> 24.3.
-                const uint32_t first = (local & 1) ? 0u : 1u;
-                const uint32_t idesc128 = (idesc & ~(0x3Fu << 17)) | (16u << 17);
-                const uint32_t stage0 = stage;
-                for (int kb = kt; kb < wu.kb1 && !aborted; ++kb) {
-                    if (!stage_ready(kb)) {
-                        aborted = true;
-                        break;
-                    }
-                    issue_mmas(wu, kb, stage, d_tmem + 128 * first, idesc128, first * kBoxRows * kAtomBytes, 4 * first);
-                    next_stage();
-                }
-                if (!aborted) {
-                    tc_commit_pair_multicast_e(e, &sm.tfull[0], both);  // the shared half is complete in both CTAs
-                    uint32_t st = stage0;
-                    for (int kb = kt; kb < wu.kb1; ++kb) {
-                        issue_mmas(wu, kb, st, d_tmem + 128 * (first ^ 1u), idesc128,
-                                   (first ^ 1u) * kBoxRows * kAtomBytes, 4 * (first ^ 1u));
-                        tc_commit_pair_multicast_e(e, &sm.empty[st], both);
-                        if (++st == kStages) st = 0;
-                    }
                 }
             }
             if (aborted) {
                 if (lane == 0) record_timeout(sm, p.status);
                 break;
             }
-            tc_commit_pair_multicast_e(e, &sm.tfull[kTail > 0 ? 1 + (local & 1) : buf], both);  // accumulator complete in both CTAs
+            tc_commit_pair_multicast_e(e, &sm.tfull[buf], both);  // accumulator complete in both CTAs
         }
         // All MMAs and copies issued by this warp complete before teardown.
         if (e) {
@@ -1111,13 +1047,6 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
                 for (int hh = 0; hh < kHalves; ++hh) {
                     const int h = hh ^ h_first;
                     const int nc = h == 0 ? 4 : (BN - 128) / 32;
-                    if (kTail > 0 && hh == 1) {  // the other half completes on its own
-                        ok = __all_sync(0xFFFFFFFFu, sm.abort_flag == 0 &&
-                                                         mbar_wait_bounded(&sm.tfull[1 + (local & 1)],
-                                                                           static_cast<uint32_t>(local >> 1) & 1u, p.wait_ns));
-                        if (!ok) break;
-                        tc_fence_after_sync();
-                    }
                     uint32_t r[4][32];
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
@@ -1168,13 +1097,6 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
                 for (int hh = 0; hh < kHalves; ++hh) {
                     const int h = hh ^ h_first;
                     const int nc = h == 0 ? 4 : (BN - 128) / 32;
-                    if (kTail > 0 && hh == 1) {  // the other half completes on its own
-                        ok = __all_sync(0xFFFFFFFFu, sm.abort_flag == 0 &&
-                                                         mbar_wait_bounded(&sm.tfull[1 + (local & 1)],
-                                                                           static_cast<uint32_t>(local >> 1) & 1u, p.wait_ns));
-                        if (!ok) break;
-                        tc_fence_after_sync();
-                    }
                     uint32_t r[4][32];
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
@@ -1206,10 +1128,6 @@ __global__ void __cluster_dims__(2 * S, 1, 1) __launch_bounds__(gemm_threads<OUT
                         ++pieces;
                     }
                 }
-            }
-            if (!ok) {
-                if (lane == 0) record_timeout(sm, p.status);
-                break;
             }
         }
         if (e) bulk_wait_group0();

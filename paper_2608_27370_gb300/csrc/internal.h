@@ -168,8 +168,7 @@ struct GemmArgs {
 
 // Tensor maps of one GEMM launch.
 //   a:   A [M, K] (128-byte swizzle, box {128 bytes, 128 rows})
-//   b:   B [N, K] (box {128 bytes, tile_n / 2 rows}: half of a tile per CTA;
-//        64 rows where a 256-wide block-scaled tile takes its half in two copies)
+//   b:   B [N, K] (box {128 bytes, tile_n / 2 rows}: half of a tile per CTA)
 //   d:   D [M, N] bf16 (64-byte swizzle, box {32, 32}); with accumulate_f32,
 //        the FP32 main-grad [M, N] (128-byte swizzle, box {32, 32})
 //   ws:  workspace [splits * splitk_rows_per_chunk(M), N] fp32 (128-byte

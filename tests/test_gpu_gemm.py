@@ -404,13 +404,12 @@ def test_dense_gemm_narrow_tiles(M, N, K, kind):
     assert_close(y, ref, kind)
 
 
-# 256-wide block-scaled tiles issue their last three k-blocks as two 128-wide
-# halves: reductions shorter than, as long as and longer than that, several
-# tiles per pair in both accumulator positions, the last column of tiles half
-# empty.
+# 256-wide block-scaled tiles, consecutive ones sharing half of their
+# accumulators: short reductions, several tiles per pair in both accumulator
+# positions, the last column of tiles half empty.
 @pytest.mark.parametrize("K", [128, 256, 384, 512, 1152])
 @pytest.mark.parametrize("main_grad", [False, True])
-def test_block_gemm_tail_halves(K, main_grad):
+def test_block_gemm_shared_accumulator_halves(K, main_grad):
     M, N = 3200, 3456  # 13 x 14 pair tiles: two or three per pair
     x, w, _ = _inputs(M, N, K, 8200 + K, t3=True)
     xq = P.quantize(x, P.E4M3, P.SCALE_BLOCK, P.ROLE_ACT, transpose=False)
@@ -426,7 +425,7 @@ def test_block_gemm_tail_halves(K, main_grad):
     torch.cuda.synchronize()
     assert P.puro_fp8_get_status(status) == 0
     A, B = (O.dequant_rows_1x128(*par_quantize_rows_1x128(bits(t), P.E4M3), P.E4M3) for t in (x, w))
-    check_gemm_every_tile(out, A, B, np.random.default_rng(8300 + K), "tail halves")
+    check_gemm_every_tile(out, A, B, np.random.default_rng(8300 + K), "shared halves")
 
 
 # A launch of one tile a pair prefetches a B of 8 MB or more while the kernel before still runs:
