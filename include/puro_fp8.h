@@ -295,8 +295,9 @@ puro_status_t puro_fp8_linear_wgrad(const puro_fp8_tensor_t *dy_t, const puro_fp
  * worth of short ones, so the pairs finish together.  A Wgrad that would
  * split its reduction with the given workspace joins the Dgrad unsplit in
  * such a launch when that is modelled faster (it is for every linear of the
- * Qwen2-1.5B and Qwen3-1.7B shapes at their token counts).  Each output of a
- * grouped launch is bit-identical to the separate call's without a
+ * Qwen2-1.5B and Qwen3-1.7B shapes at their token counts) and N > 256; up to
+ * N = 256 it keeps the split on most shapes, for the shorter FP32 sums.  Each
+ * output of a grouped launch is bit-identical to the separate call's without a
  * workspace.  Otherwise (per-tensor scaling, a split reduction, the
  * 224-wide tile form, an empty extent) the two GEMMs are launched one after
  * the other, exactly as the separate entry points would.  Arguments as for
@@ -411,7 +412,7 @@ size_t puro_fp8_scale_bytes(int64_t rows, int64_t red);
 /*
  * Scratch bytes that let a GEMM with output [rows_out, cols_out] and
  * reduction extent `red` use its split-reduction schedule (0 if it never
- * would): splits * ceil(rows_out/128)*128 * cols_out * 4.  Host-only, no
+ * would): splits * ceil(rows_out/256)*256 * cols_out * 4.  Host-only, no
  * CUDA call.
  */
 size_t puro_fp8_workspace_size(int64_t rows_out, int64_t cols_out, int64_t red);

@@ -132,13 +132,16 @@ puro_status_t prepare_fp8_gemm(const puro_fp8_tensor_t *a, const puro_fp8_tensor
     const bool block = a->scaling == PURO_SCALE_BLOCK;
 
     // Split the reduction across CTA pairs when the output has too few tiles
-    // to fill the GPU and the caller supplied enough aligned scratch;
-    // otherwise the block-scaled kind picks its tile width.
+    // to fill the GPU and the caller supplied enough aligned scratch (which
+    // the split inside clusters then leaves alone).
     const int sp = choose_splits(M, N, K, false);
     const bool split = sp > 1 && workspace && aligned16(workspace) &&
                        workspace_bytes >= splitk_workspace_bytes(M, N, K, false);
     const int cluster = split ? cluster_split(M, N, K, sp) : 1;
-    const int tile_n = cluster > 1 ? 128 : split ? 256 : width ? width : tile_width(block ? kGemmFP8Block : kGemmFP8Tensor, accumulate_f32, M, N, K);
+    const int tile_n = cluster > 1 ? 128
+                       : split     ? 256
+                       : width     ? width
+                                   : tile_width(block ? kGemmFP8Block : kGemmFP8Tensor, accumulate_f32, M, N, K);
 
     GemmMaps m{};
     if (!make_map(&m.a, CU_TENSOR_MAP_DATA_TYPE_UINT8, a->data, K, M, K, kGemmBKBytes, kGemmBM,
@@ -212,7 +215,7 @@ puro_status_t fp8_gemm(const puro_fp8_tensor_t *a, const puro_fp8_tensor_t *b, v
 // block-scaled) runs, given `ws` usable workspace bytes: one grouped launch
 // when both GEMMs are unsplit -- or when the Wgrad would split
 // its reduction but one grouped launch with it unsplit is modelled faster --
-// else each GEMM on its own (a split Wgrad adds its reduction kernel).
+// else each GEMM on its own (one split through memory adds its reduction kernel).
 struct BackwardPlan {
     bool grouped;        // one launch for both
     bool wgrad_unsplit;  // the Wgrad gives up the split it would take, to join the Dgrad

@@ -11,8 +11,8 @@
 
 namespace puro {
 
-// Launch `kern` on `s` with programmatic stream serialisation (the kernel
-// calls pdl_wait() before touching global memory; see ptx.cuh).
+// Launch `kern` on `s` with programmatic stream serialisation: it starts while
+// the kernel before runs and waits for it itself (pdl_wait(); see ptx.cuh).
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                               Args &&...args) {
@@ -137,24 +137,25 @@ struct GemmArgs {
     GemmKind kind;
     int a_fmt, b_fmt;            // FP8 formats (0 = E4M3, 1 = E5M2)
     int64_t M, N, K;
-    int tile_n;                  // 256, 192 or 128 (see choose_tile_n), or 224 (block kind, BF16 out, forced); split: 256
+    int tile_n;                  // 256, 192 or 128 (see choose_tile_n), or 224 (block kind, BF16 out,
+                                 // forced); split: 256 through memory, 128 in clusters
+    const uint8_t *b;            // FP8 kinds: B's codes (prefetched by launches of one tile a pair)
     // kGemmFP8Block: scale vectors of B (the 224-wide form gathers them
     // itself; the others load them through GemmMaps::sfb).
-    const uint8_t *b;            // FP8 kinds: B's codes
     const uint8_t *sfb;
     // kGemmFP8Tensor: dequantisation factors of A and B.
     const float *sia, *sib;
     int32_t *status;             // optional device status word
     uint64_t wait_timeout_ns;
     int num_sms;
-    // split reduction (FP8 kinds only): splits > 1 needs `workspace` of
-    // splitk_workspace_bytes(M, N, K) bytes; `out` is D (bf16)
+    // split reduction (FP8 kinds only): splits > 1 with cluster == 1 needs
+    // `workspace` of splitk_workspace_bytes(M, N, K) bytes; `out` is D
     int splits;
     int cluster;                 // splits > 1: pairs of a cluster that share the reduction on chip (2 or 4), or 1
     void *workspace;
     void *out;
     // out is an FP32 main-grad [M, N] that receives out += A * B^T (block
-    // or per-tensor kinds; 256-wide tiles)
+    // or per-tensor kinds)
     bool accumulate_f32;
     // kGemmOutQuant (block kind): the epilogue quantises bf16(D) into the
     // rowwise copy q [M, N] (scales q_scale) and, when qt is set, the
@@ -172,7 +173,7 @@ struct GemmArgs {
 //   d:   D [M, N] bf16 (64-byte swizzle, box {32, 32}); with accumulate_f32,
 //        the FP32 main-grad [M, N] (128-byte swizzle, box {32, 32})
 //   ws:  workspace [splits * splitk_rows_per_chunk(M), N] fp32 (128-byte
-//        swizzle, box {32, 32}); only read when g.splits > 1
+//        swizzle, box {32, 32}); only read when split through memory
 //   sfa, sfb (kGemmFP8Block only): the scale vectors of A / B,
 //        [rows/128][ceil(K/512)][512] bytes viewed as uint32
 //        [rows/128 * ceil(K/512), 128], box {128, 1}

@@ -1,7 +1,7 @@
 // ptx.cuh -- thin inline-PTX wrappers for sm_103a (Blackwell) used by the
 // quantise and GEMM kernels: mbarriers, TMA (cp.async.bulk.tensor), bulk
 // copies, and the tcgen05 tensor-core / tensor-memory instructions.
-// Every wrapper is one documented PTX instruction (PTX ISA 8.7+).
+// Every wrapper is one documented PTX instruction (PTX ISA 8.7+) or a few.
 #pragma once
 
 #include <cuda.h>
@@ -13,12 +13,6 @@ namespace puro {
 
 PURO_DEV uint32_t smem_u32(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-PURO_DEV uint32_t lane_id() {
-    uint32_t l;
-    asm volatile("mov.u32 %0, %%laneid;" : "=r"(l));
-    return l;
 }
 
 // 1 in one lane of the warp (always the same one), 0 in the others.  The forms
@@ -41,8 +35,13 @@ PURO_DEV uint64_t global_timer_ns() {
 // start (and run its prologue: barrier set-up, tensor-memory allocation,
 // descriptor prefetch) while the previous kernel on the stream finishes.
 // pdl_wait() blocks until the previous kernels have completed and their
-// memory is visible; every kernel calls it before its first global-memory
-// access, then pdl_launch_dependents() lets the next kernel start launching.
+// memory is visible; every kernel calls it before it writes global memory and
+// before it reads any that the kernel just before may write, and only then
+// pdl_launch_dependents(), which lets the next kernel start launching.  So what
+// the kernel before the previous one wrote is complete when a kernel starts.
+// Two accesses come before the wait: the RMSNorm quantiser's first tile of h
+// (see launch_quantize_rmsnorm) and the GEMM's prefetch of B into L2, which
+// delivers nothing.
 PURO_DEV void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 PURO_DEV void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -85,10 +84,6 @@ PURO_DEV void fence_proxy_async_smem() {
 PURO_DEV void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                  : "memory");
-}
-
-PURO_DEV void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 PURO_DEV bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
@@ -188,17 +183,6 @@ PURO_DEV void bulk_wait_group_read() { asm volatile("cp.async.bulk.wait_group.re
 // Wait until all committed bulk stores are complete.
 PURO_DEV void bulk_wait_group0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-// ------------------------------------------------------- Ampere cp.async
-// 16-byte global -> shared copy; src_bytes < 16 zero-fills the remainder.
-PURO_DEV void cp_async_16(void *dst, const void *src, uint32_t src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)),
-                 "l"(reinterpret_cast<uint64_t>(src)), "r"(src_bytes)
-                 : "memory");
-}
-PURO_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-PURO_DEV void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // ------------------------------------------------------------- tcgen05
 // Tensor memory: 128 lanes x 512 columns of 32-bit cells per SM.  An
 // address is (lane << 16) | column.
@@ -224,12 +208,8 @@ PURO_DEV void st_cluster_v4(uint32_t addr, const uint4 &v) {
                  : "memory");
 }
 
-// All threads of all CTAs of the cluster (release / acquire).
-PURO_DEV void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// The two halves of cluster_sync, for work in between.
+// Barrier of all threads of all CTAs of the cluster (release / acquire), in two
+// halves for work in between.
 PURO_DEV void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 PURO_DEV void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
@@ -259,7 +239,6 @@ PURO_DEV void mbar_arrive_cluster_cta_scope(uint32_t bar_cluster) {
 
 // 2-D tiled load into this CTA's shared memory whose completion is counted
 // on an mbarrier that may live in the peer CTA of the pair.
-
 PURO_DEV void tma_load_2d_pair_e(uint32_t e, void *dst, const CUtensorMap *map, uint32_t bar_cluster, int32_t x,
                                  int32_t y) {
     asm volatile(
@@ -294,21 +273,6 @@ PURO_DEV void tc_commit_pair(uint64_t *bar) {
                      smem_u32(bar))
                  : "memory");
 }
-// The same, arriving on `bar` in every cluster CTA of `cta_mask`.
-
-// Pair MMA D(tmem) (+)= A(smem) * B(smem)^T, kind::f16 (bf16/fp16 inputs,
-// f32 accumulate).
-
-// kind::f8f6f4 (e4m3/e5m2 inputs, f32 accumulate), no block scaling.
-
-// kind::mxf8f6f4 with one UE8M0 scale per 32 elements of K for each row of
-// A and of B (scale_vec::1X); the scales are read from tensor memory (each
-// CTA's own: its 128 rows of A, all N rows of B).
-
-// Copy 32 rows x 128 bits from shared memory into tensor memory, replicated
-// into each of the four 32-lane quarters (warpx4): row r lands in lane r of
-// every quarter, its four 32-bit words in columns taddr .. taddr+3.  The
-// pair form copies each CTA's shared memory into its own tensor memory.
 
 // Each thread of the warp reads 32 consecutive 32-bit columns of its own
 // lane (warp w may address lanes 32*(w%4) .. 32*(w%4)+31 only).
@@ -327,6 +291,8 @@ PURO_DEV void tmem_ld_32x32b_x32(uint32_t taddr, uint32_t (&r)[32]) {
 }
 PURO_DEV void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// Pair MMA D(tmem) (+)= A(smem) * B(smem)^T, kind::f16 (bf16/fp16 inputs,
+// f32 accumulate).
 PURO_DEV void mma_pair_f16_e(uint32_t e, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                              uint32_t accumulate) {
     asm volatile(
@@ -335,6 +301,7 @@ PURO_DEV void mma_pair_f16_e(uint32_t e, uint32_t d_tmem, uint64_t adesc, uint64
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(e)
         : "memory");
 }
+// kind::f8f6f4 (e4m3/e5m2 inputs, f32 accumulate), no block scaling.
 PURO_DEV void mma_pair_f8_e(uint32_t e, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                             uint32_t accumulate) {
     asm volatile(
@@ -343,6 +310,9 @@ PURO_DEV void mma_pair_f8_e(uint32_t e, uint32_t d_tmem, uint64_t adesc, uint64_
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(e)
         : "memory");
 }
+// kind::mxf8f6f4 with one UE8M0 scale per 32 elements of K for each row of
+// A and of B (scale_vec::1X); the scales are read from tensor memory (each
+// CTA's own: its 128 rows of A, all N rows of B).
 PURO_DEV void mma_pair_mxf8_e(uint32_t e, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                               uint32_t sfa_tmem, uint32_t sfb_tmem, uint32_t accumulate) {
     asm volatile(
@@ -352,6 +322,10 @@ PURO_DEV void mma_pair_mxf8_e(uint32_t e, uint32_t d_tmem, uint64_t adesc, uint6
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(sfa_tmem), "r"(sfb_tmem), "r"(e)
         : "memory");
 }
+// Copy 32 rows x 128 bits from shared memory into tensor memory, replicated
+// into each of the four 32-lane quarters (warpx4): row r lands in lane r of
+// every quarter, its four 32-bit words in columns taddr .. taddr+3.  The
+// pair form copies each CTA's shared memory into its own tensor memory.
 PURO_DEV void tmem_cp_pair_32x128b_warpx4_e(uint32_t e, uint32_t taddr, uint64_t sdesc) {
     asm volatile(
         "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q tcgen05.cp.cta_group::2.32x128b.warpx4 [%0], %1;\n\t}" ::"r"(
@@ -359,6 +333,7 @@ PURO_DEV void tmem_cp_pair_32x128b_warpx4_e(uint32_t e, uint32_t taddr, uint64_t
         "l"(sdesc), "r"(e)
         : "memory");
 }
+// tc_commit_pair arriving on `bar` in every cluster CTA of `cta_mask`.
 PURO_DEV void tc_commit_pair_multicast_e(uint32_t e, uint64_t *bar, uint16_t cta_mask) {
     asm volatile(
         "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
@@ -384,20 +359,6 @@ PURO_DEV uint64_t smem_desc_k_sw128(uint32_t saddr) {
     d |= static_cast<uint64_t>(1024 >> 4) << 32;
     d |= static_cast<uint64_t>(1) << 46;
     d |= static_cast<uint64_t>(2) << 61;
-    return d;
-}
-
-// The same for a tile whose K rows are kRowBytes (128 or 64) bytes, written by
-// TMA with the matching swizzle: 8-row atoms of 8 * kRowBytes bytes.
-template <int kRowBytes>
-PURO_DEV uint64_t smem_desc_k_swizzled(uint32_t saddr) {
-    static_assert(kRowBytes == 128 || kRowBytes == 64, "128- or 64-byte swizzle");
-    uint64_t d = 0;
-    d |= static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
-    d |= static_cast<uint64_t>(1) << 16;
-    d |= static_cast<uint64_t>((8 * kRowBytes) >> 4) << 32;
-    d |= static_cast<uint64_t>(1) << 46;
-    d |= static_cast<uint64_t>(kRowBytes == 128 ? 2 : 4) << 61;  // 2: 128-byte swizzle, 4: 64-byte swizzle
     return d;
 }
 

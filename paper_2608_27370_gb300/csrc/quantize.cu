@@ -146,6 +146,7 @@ PURO_DEV float row_rstd(const uint4 *row, int64_t n8, int64_t cols, float eps, i
 }
 
 // rstd of each row of h [rows, cols] (cols a multiple of 8), one warp per row.
+// The trigger must stay behind the wait: see launch_quantize_rmsnorm.
 __global__ void __launch_bounds__(256) rmsnorm_rstd_kernel(const uint16_t *__restrict__ h, int64_t rows, int64_t cols,
                                                            float eps, float *__restrict__ rstd) {
     pdl_wait();
@@ -625,7 +626,6 @@ PURO_DEV uint2 swiglu_chunk4(uint2 g, uint2 u) {
     return make_uint2(out[0], out[1]);
 }
 
-//
 // Behind a producer the kernel is bound by its instructions between the tile's
 // three barriers, not by HBM, so the produced block stays in registers (it is
 // written back to shared memory only for a y output), RMSNorm's products are
@@ -1144,6 +1144,9 @@ static cudaError_t launch_rms_f(const QuantArgs &a, const CUtensorMap &tm_x, con
                    : launch_quant_t<FMT, kQuantBlockAct, false, kProdRmsNorm>(a, tm_x, tm_q, tm_qt, s, &tm_y, prod);
 }
 
+// To be launched directly behind launch_rmsnorm_rstd on the same h: the quantiser
+// loads its first tile of h before its own wait (see quant_act_kernel), and it is
+// the rstd pass's wait, ahead of its trigger, that makes h whole by then.
 cudaError_t launch_quantize_rmsnorm(const QuantArgs &a, const CUtensorMap &tm_x, const CUtensorMap &tm_q,
                                     const CUtensorMap &tm_qt, const CUtensorMap &tm_y, const ProdArgs &prod,
                                     cudaStream_t s) {
